@@ -14,10 +14,10 @@
 // (fused with the projector pass of G) and one for the update, plus a second
 // pair of passes only when the update cancelled the vector to below 1e-2 of
 // its norm (the Daniel-Gragg-Kaufman-Stewart test with a loose threshold).
-// GB300 runs FP64 at about 1/64 of its FP32 rate, so these vector kernels
-// are bound by FP64 instructions rather than by HBM: each keeps the FP64
-// work per element at 4 multiply-adds per basis vector and pass, and in the
-// precision form the projector (part of applying G) runs in FP32.  The
+// GB300 runs FP64 at about 1/64 of its FP32 rate, so the sums and products of
+// these passes run on the integer pipe (fixed64.cuh) on a basis stored for it
+// (KrylovBasis), and in the precision form the projector (part of applying G)
+// runs in FP32.  The
 // Hessenberg matrix and the norms stay on the device; the host waits once
 // per substep, after the candidate substep exponentials are evaluated.
 #include <algorithm>
@@ -26,6 +26,7 @@
 
 #include "afem_internal.h"
 #include "arnoldi.cuh"
+#include "fixed64.cuh"
 #include "vec_common.cuh"
 
 namespace afem {
@@ -232,340 +233,656 @@ __global__ void __launch_bounds__(kRedThreads) overlap32_kernel(const float2* __
     }
 }
 
-// acc[2i], acc[2i+1] += conj(u_i) mx (i < NV) and acc[2NV] += conj(x) mx, with
-// mx = m x formed once: 4 FP64 multiply-adds per basis vector.
-template <int NV>
-__device__ __forceinline__ void accumulate_dots(double (&acc)[2 * NV + 1], const double2 (&u)[NV > 0 ? NV : 1],
-                                                double2 x, double m) {
-    const double2 mx = make_double2(m * x.x, m * x.y);
+// Krylov vectors are stored as integers (KrylovBasis below) and unscaled: V_0 is
+// the substep's start vector and V_{i+1} the raw Gram-Schmidt remainder of the cell
+// pass applied to V_i, with q_i = f[i] V_i, f[0] = 1 / beta, f[i] = f[i-1] / h_{i,i-1}
+// (= 1 / |V_i|_M; 0 after a breakdown, h <= 1e-14 beta), so no pass over the basis
+// only to scale it and no scaling of the new vector.  The pass that finishes
+// V_i writes f[i] (and f[kScaleBeta] = beta); as a chain of float64 divisions by
+// one thread of every block of every pass it took 6 us at 12 vectors.
+constexpr int kScaleBeta = kMaxKrylov + 1;
+
+// ------------------------------------------------- the Krylov basis in integers
+// The Gram-Schmidt passes read every basis vector twice per new vector and are
+// products and sums of float64 numbers, which run on the integer pipe
+// (fixed64.cuh).  The vectors are therefore stored ready for it: per group of
+// rows one exponent e (of the largest component), and per component the
+// integer X = v 2^(1082 - e), |X| < 2^60, split h 2^32 + l,
+// as (re l, re h, im l, im h): 16 bytes, as the float64 pair was, and seven
+// bits finer than float64 at the group's largest component.  Reading a
+// component then costs no conversion.  Measured on 10 vectors of 775,009 x 4
+// (499 MB, 73 us at the copy rate): inner products with the projector 259 us as
+// FP64 multiply-adds, 237 us converting from float64 on the way, 127 us stored
+// as integers; the update 245 / 154 / 109 us, the close of a substep 254 / 103 us.
+// What bounds them now is instruction issue (about 50 per element and vector, 12
+// of them IMAD.WIDE at 31 lanes per clock) beside 55-70 % of the copy rate.
+//
+// Thread t < n R of a 256-thread block (R = 256 / n) owns column p = t % n and,
+// in tile T, the rows T E R + r + R e (e < E, r = t / n): a group, the rows that
+// one thread sums together, with one exponent (4 bytes beside 16 E of data), so
+// that no thread waits for another's scale.  Storage follows the threads, not
+// the rows: element (T, e, t) of a vector, exponent (T, t).  E (4, 2 or 1) is chosen per call so
+// that the tiles fill the chip (krylov_rows).  Exponent 0: all components zero;
+// 0x7FF: the group holds a non-finite value.
+constexpr int kFxNan = 0x7FF;
+
+__device__ __forceinline__ Fx fx_re(int4 v) { return Fx{v.y, v.x}; }
+__device__ __forceinline__ Fx fx_im(int4 v) { return Fx{v.w, v.z}; }
+
+struct TileRows {
+    int p, r, R;
+    bool active;
+    __device__ __forceinline__ TileRows(int n) {
+        R = kRedThreads / n;
+        active = int(threadIdx.x) < n * R;
+        r = active ? int(threadIdx.x) / n : 0;
+        p = active ? int(threadIdx.x) - r * n : 0;
+    }
+};
+
+// The basis vectors of a block's tiles as one stream of (tile, vector) items,
+// item q = vector q % nv of the block's tile q / nv: each thread copies its own
+// E rows of the item kStages - 1 ahead into its own slots of shared memory
+// (cp.async, no barrier), so that about 50 KB per SM are in flight whatever the
+// registers allow.  Loads into registers one vector ahead kept 32 KB in flight
+// and ran at 4.5 TB/s.
+__device__ __forceinline__ void copy16(void* smem_dst, const void* gmem_src) {
+    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void copy4(void* smem_dst, const void* gmem_src) {
+    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void copy_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(LEFT) : "memory");
+}
+
+template <int E, int STAGES>
+struct BasisStream {
+    const int4* v;        // next item's first row
+    const int* e;         // its exponent
+    int4* slots;          // this thread's slots, [STAGES][E][kRedThreads]
+    int* eslots;          // [STAGES][kRedThreads] (STAGE_E)
+    int64_t stride, estride, wrap, ewrap;   // to the next vector; from the last vector to the next tile's first
+    int left, nv;         // tiles left, vectors
+    int i, stage;
+    __device__ __forceinline__ BasisStream(const KrylovBasis& B, int nv_, int4* sl, int* esl)
+        : v(B.V + int64_t(blockIdx.x) * (E * kRedThreads) + threadIdx.x),
+          e(B.e + int64_t(blockIdx.x) * kRedThreads + threadIdx.x), slots(sl + threadIdx.x), eslots(esl + threadIdx.x),
+          stride(B.stride), estride(B.estride), wrap(int64_t(gridDim.x) * (E * kRedThreads) - (nv_ - 1) * B.stride),
+          ewrap(int64_t(gridDim.x) * kRedThreads - (nv_ - 1) * B.estride),
+          left(int((B.tiles - blockIdx.x + gridDim.x - 1) / gridDim.x)), nv(nv_), i(0), stage(0) {}
+    template <bool STAGE_E>
+    __device__ __forceinline__ void issue() {
+        if (left > 0) {
+            int4* d = slots + stage * (E * kRedThreads);
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        acc[2 * i] = fma(u[i].x, mx.x, fma(u[i].y, mx.y, acc[2 * i]));
-        acc[2 * i + 1] = fma(u[i].x, mx.y, fma(-u[i].y, mx.x, acc[2 * i + 1]));
-    }
-    // the norm only without basis vectors; with them finish_dots takes the
-    // in-span part of the norm from the inner products (no FP64 work per element)
-    if constexpr (NV == 0) acc[0] = fma(x.x, mx.x, fma(x.y, mx.y, acc[0]));
-}
-
-// Krylov vectors are stored unscaled: V_0 is the substep's start vector and
-// V_{i+1} the raw Gram-Schmidt remainder of the cell pass applied to V_i, with
-// q_i = s_f[i] V_i, s_f[0] = 1 / beta, s_f[i] = s_f[i-1] / h_{i,i-1} (= 1 / |V_i|_M),
-// so no pass over the basis only to scale it and no FP64 scaling of the new
-// vector (0 after a breakdown, h <= 1e-14 beta).  Callers __syncthreads()
-// before use.
-__device__ __forceinline__ void krylov_scales(const double2* __restrict__ H, int ldh,
-                                              const double2* __restrict__ beta2, int nv, double* s_f) {
-    if (threadIdx.x != 0 || nv <= 0) return;
-    const double beta = sqrt(fmax(beta2->x, 0.0));
-    double f = beta > 0.0 ? 1.0 / beta : 0.0;
-    s_f[0] = f;
-    for (int i = 1; i < nv; ++i) {
-        const double h = H[(i - 1) * ldh + i].x;
-        f = (h > 1e-14 * beta && h > 0.0) ? f / h : 0.0;
-        s_f[i] = f;
-    }
-}
-
-// The block sums of acc (inner products of the raw vector w with the stored
-// V_i), then in the last block the true values for the vector fw w with
-// fw = s_f[NV-1] (1 when NV = 0): out[i] = s_f[i] fw (acc[2i], acc[2i+1]) =
-// <q_i, fw w> for i < NV and out[NV] = (sum_i |out[i]|^2, 0), the squared
-// norm of the part of fw w in the span of q_0..q_{NV-1} (for NV = 0,
-// |w|^2 itself).  By Pythagoras the norm before the update is this plus the
-// norm the update leaves, which is how the re-orthogonalisation test uses it.
-template <int NV>
-// Returns true in the last block (after every block has finished its reads).
-__device__ __forceinline__ bool finish_dots(double (&acc)[2 * NV + 1], const double* s_f,
-                                            double* __restrict__ partial, unsigned* __restrict__ counter,
-                                            double2* __restrict__ out) {
-    constexpr int CNT = NV > 0 ? 2 * NV : 1;
-    block_row_partial<2 * NV + 1>(acc, CNT, partial);
-    __shared__ double s_sum[kRedThreads];
-    if (!last_block_sum(partial, CNT, counter, s_sum)) return false;
-    const double fw = NV > 0 ? s_f[NV > 0 ? NV - 1 : 0] : 1.0;
-    for (int i = threadIdx.x; i < NV; i += blockDim.x) {
-        const double f = s_f[i] * fw;
-        out[i] = make_double2(f * s_sum[2 * i], f * s_sum[2 * i + 1]);
-    }
-    if (threadIdx.x == 0) {
-        double nn = 0.0;
-        if (NV == 0) {
-            nn = s_sum[0];
-        } else {
-            for (int i = 0; i < NV; ++i) {
-                const double f = s_f[i] * fw;
-                nn += f * f * (s_sum[2 * i] * s_sum[2 * i] + s_sum[2 * i + 1] * s_sum[2 * i + 1]);
+            for (int r = 0; r < E; ++r) copy16(d + r * kRedThreads, v + r * kRedThreads);
+            if (STAGE_E) copy4(eslots + stage * kRedThreads, e);
+            const bool last = ++i == nv;
+            v += last ? wrap : stride;
+            if (STAGE_E) e += last ? ewrap : estride;
+            if (last) {
+                i = 0;
+                --left;
             }
         }
-        out[NV] = make_double2(nn, 0.0);
+        copy_commit();
+        stage = stage + 1 == STAGES ? 0 : stage + 1;
     }
-    return true;
-}
+};
 
-// Gram-Schmidt inner products: out[i] = <q_i, w>_M for i < NV and out[NV] as
-// finish_dots states, over interior rows.  Skipped when gate && !*gate.
-// NV is a template parameter so that the NV + 1 loads of a row are issued
-// back to back before any of them is used.
-template <int NV>
-__global__ void __launch_bounds__(kRedThreads) krylov_dots_kernel(
-    const double2* __restrict__ w, const double2* __restrict__ V, int64_t stride, const double* __restrict__ ml,
-    int64_t n_int, int n, const int* __restrict__ gate, const double2* __restrict__ H, int ldh,
-    const double2* __restrict__ beta2, double* __restrict__ partial, unsigned* __restrict__ counter,
-    double2* __restrict__ out) {
-    if (gate && *gate == 0) return;
-    __shared__ double s_f[NV > 0 ? NV : 1];
-    if (NV > 0) krylov_scales(H, ldh, beta2, NV, s_f);
-    double acc[2 * NV + 1];
-#pragma unroll
-    for (int i = 0; i < 2 * NV + 1; ++i) acc[i] = 0.0;
-    const RowCol rc(n);
-    if (rc.active) {
-        for (int64_t k = int64_t(blockIdx.x) * rc.R + rc.r; k < n_int; k += int64_t(gridDim.x) * rc.R) {
-            const int64_t o = k * n + rc.p;
-            const double m = ml[k];
-            const double2 x = w[o];
-            double2 u[NV > 0 ? NV : 1];
-#pragma unroll
-            for (int i = 0; i < NV; ++i) u[i] = V[i * stride + o];
-            accumulate_dots<NV>(acc, u, x, m);
-        }
-    }
-    finish_dots<NV>(acc, s_f, partial, counter, out);
-}
+// Gram-Schmidt inner products, with (MODE 1, 2) the projector pass of G in front:
+//   MODE 0: w = V_nv, the stored remainder of the first pass (second pass;
+//     skipped when gate && !*gate);
+//   MODE 1: z is the FP64 cell pass applied to V_{nv-1}, and
+//     w[k][p] = ML^-1[k] z[k][p] - sum_j phi[k][j] S[j][p] on interior rows
+//     (0 on the others), which is G q_{nv-1} / s_f[nv-1], is written to wd;
+//   MODE 2: the same for the precision form, the projector in FP32 from the
+//     complex64 cell-pass output and orbitals; w is a complex64 vector (times
+//     2^kv, see below) and replaces the cell pass's output in place.
+// out[i] = s_f[i] fw sum_k m_k conj(V_i) w = <q_i, fw w>_M for i < nv with
+// fw = s_f[nv-1], and out[nv] = (sum_i |out[i]|^2, 0), the squared norm of the
+// part of fw w in the span of q_0..q_{nv-1}: by Pythagoras the norm before the
+// update is this plus the norm that the update leaves, which is how the
+// re-orthogonalisation test uses it.
+//
+// A thread forms m w of its E rows on their common scale and walks the basis
+// vectors: E staged rows, 12 E IMAD.WIDE and two float64 additions into its sums
+// in shared memory.
+struct GsDotsArgs {
+    const double2* z;
+    float2* z32;
+    const double2* phi;
+    const float2* phi32;
+    const double2* S;
+    double* S_slots;        // MODE 2: overlap32_kernel's slots (cleared by the last block), or null
+    const double* ml_inv;
+    const float* ml_inv32;
+    const double* ml;
+    int64_t n_int, N;
+    int n;
+    double2* wd;
+    KrylovBasis B;
+    int nv;
+    const int* gate;
+    const double* f;        // the basis's scales
+    double* partial;
+    unsigned* counter;
+    double2* out;
+};
 
-// The projector pass of G fused with the first Gram-Schmidt pass (FP64 form):
-// z is the cell pass applied to the stored V_{NV-1}, so the raw vector
-// w[k][p] = ML^-1[k] z[k][p] - sum_j phi[k][j] S[j][p] on interior rows (0 on
-// the others) is G q_{NV-1} / s_f[NV-1]; it is written unscaled, and
-// out[i] = <q_i, G q_{NV-1}>_M (i < NV) and out[NV] (see finish_dots) are
-// formed from the values in registers, so w is not read back.
-template <int NV>
-__global__ void __launch_bounds__(kRedThreads) project_dots_kernel(
-    const double2* __restrict__ z, const double2* __restrict__ phi, const double2* __restrict__ S,
-    const double* __restrict__ ml_inv, const double* __restrict__ ml, int64_t n_int, int64_t N, int n,
-    double2* __restrict__ w, const double2* __restrict__ V, int64_t stride, const double2* __restrict__ H, int ldh,
-    const double2* __restrict__ beta2, double* __restrict__ partial, unsigned* __restrict__ counter,
-    double2* __restrict__ out) {
-    __shared__ double2 s_S[kMaxOrbProj * kMaxOrbProj];
-    __shared__ double s_f[NV];
-    for (int i = threadIdx.x; i < n * n; i += blockDim.x) s_S[i] = S[i];
-    krylov_scales(H, ldh, beta2, NV, s_f);
-    __syncthreads();
-    double acc[2 * NV + 1];
-#pragma unroll
-    for (int i = 0; i < 2 * NV + 1; ++i) acc[i] = 0.0;
-    const RowCol rc(n);
-    if (rc.active) {
-        const int p = rc.p;
-        for (int64_t k = int64_t(blockIdx.x) * rc.R + rc.r; k < N; k += int64_t(gridDim.x) * rc.R) {
-            const int64_t o = k * n + p;
-            double2 x = make_double2(0.0, 0.0);
-            if (k < n_int) {
-                double2 u[NV];
-#pragma unroll
-                for (int i = 0; i < NV; ++i) u[i] = V[i * stride + o];
-                const double s = ml_inv[k];
-                const double2 zo = z[o];
-                x = make_double2(zo.x * s, zo.y * s);
-                for (int j = 0; j < n; ++j) {
-                    const double2 f = phi[k * n + j];
-                    const double2 c = s_S[j * n + p];
-                    x.x = fma(-f.x, c.x, fma(f.y, c.y, x.x));
-                    x.y = fma(-f.x, c.y, fma(-f.y, c.x, x.y));
+template <int E, int MODE, int STAGES>
+__global__ void __launch_bounds__(kRedThreads, 2) gs_dots_kernel(const __grid_constant__ GsDotsArgs a) {
+    if (MODE == 0 && a.gate && *a.gate == 0) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double2* s_acc = reinterpret_cast<double2*>(smem_raw);                  // [nv][kRedThreads]
+    int4* s_v = reinterpret_cast<int4*>(s_acc + a.nv * kRedThreads);       // [STAGES][E][kRedThreads]
+    int* s_ve = reinterpret_cast<int*>(s_v + STAGES * E * kRedThreads);    // [STAGES][kRedThreads]
+    __shared__ double s_f[kMaxKrylov];
+    __shared__ double2 s_S[MODE == 1 ? kMaxOrbProj * kMaxOrbProj : 1];
+    __shared__ float2 s_S32[MODE == 2 ? kMaxOrbProj * kMaxOrbProj : 1];
+    const int nv = a.nv, n = a.n, tid = threadIdx.x;
+    for (int i = 0; i < nv; ++i) s_acc[i * kRedThreads + tid] = make_double2(0.0, 0.0);
+    if constexpr (MODE == 1)
+        for (int i = tid; i < n * n; i += blockDim.x) s_S[i] = a.S[i];
+    if constexpr (MODE == 2) {
+        // the overlaps: the sum of overlap32_kernel's slots, or S itself (zero
+        // without the projector)
+        for (int i = tid; i < n * n; i += blockDim.x) {
+            double2 v = make_double2(0.0, 0.0);
+            if (a.S_slots) {
+                for (int sl = 0; sl < kOvSlots; ++sl) {
+                    v.x += a.S_slots[sl * 2 * n * n + 2 * i];
+                    v.y += a.S_slots[sl * 2 * n * n + 2 * i + 1];
                 }
-                accumulate_dots<NV>(acc, u, x, ml[k]);
-            }
-            w[o] = x;
-        }
-    }
-    finish_dots<NV>(acc, s_f, partial, counter, out);
-}
-
-// The same for the precision form: the projector in FP32 from the complex64
-// cell-pass output z and the complex64 orbitals phi32 (part of applying G),
-// the result widened to FP64 for the Gram-Schmidt inner products.
-template <int NV>
-__global__ void __launch_bounds__(kRedThreads) project32_dots_kernel(
-    const float2* __restrict__ z, const float2* __restrict__ phi, const double2* __restrict__ S,
-    const float* __restrict__ ml_inv, const double* __restrict__ ml, int64_t n_int, int64_t N, int n,
-    double2* __restrict__ w, const double2* __restrict__ V, int64_t stride, const double2* __restrict__ H, int ldh,
-    const double2* __restrict__ beta2, double* __restrict__ partial, unsigned* __restrict__ counter,
-    double2* __restrict__ out, double* __restrict__ S_slots) {
-    __shared__ float2 s_S[kMaxOrbProj * kMaxOrbProj];
-    __shared__ double s_f[NV];
-    // the overlaps: the sum of overlap32_kernel's slots (cleared by the last
-    // block below), or S itself (zero without the projector)
-    for (int i = threadIdx.x; i < n * n; i += blockDim.x) {
-        if (S_slots) {
-            double x = 0.0, y = 0.0;
-            for (int sl = 0; sl < kOvSlots; ++sl) {
-                x += S_slots[sl * 2 * n * n + 2 * i];
-                y += S_slots[sl * 2 * n * n + 2 * i + 1];
-            }
-            s_S[i] = make_float2(narrow_f64(x), narrow_f64(y));
-        } else {
-            s_S[i] = make_float2(narrow_f64(S[i].x), narrow_f64(S[i].y));
-        }
-    }
-    krylov_scales(H, ldh, beta2, NV, s_f);
-    __syncthreads();
-    // the complex64 input of the cell pass was 2^kv V_{NV-1} (krylov_update_kernel's
-    // scaling; V_0 unscaled), so the raw vector is the result times 2^-kv
-    const int kv = (NV >= 2 && s_f[NV >= 2 ? NV - 2 : 0] > 0.0) ? ilogb(s_f[NV >= 2 ? NV - 2 : 0]) : 0;
-    double acc[2 * NV + 1];
-#pragma unroll
-    for (int i = 0; i < 2 * NV + 1; ++i) acc[i] = 0.0;
-    const RowCol rc(n);
-    if (rc.active) {
-        const int p = rc.p;
-        for (int64_t k = int64_t(blockIdx.x) * rc.R + rc.r; k < N; k += int64_t(gridDim.x) * rc.R) {
-            const int64_t o = k * n + p;
-            double2 x = make_double2(0.0, 0.0);
-            if (k < n_int) {
-                double2 u[NV];
-#pragma unroll
-                for (int i = 0; i < NV; ++i) u[i] = V[i * stride + o];
-                const float s = ml_inv[k];
-                const float2 zo = z[o];
-                float2 xf = make_float2(zo.x * s, zo.y * s);
-                for (int j = 0; j < n; ++j) {
-                    const float2 f = phi[k * n + j];
-                    const float2 c = s_S[j * n + p];
-                    xf.x = fmaf(-f.x, c.x, fmaf(f.y, c.y, xf.x));
-                    xf.y = fmaf(-f.x, c.y, fmaf(-f.y, c.x, xf.y));
-                }
-                x = make_double2(widen_f32_scaled(xf.x, -kv), widen_f32_scaled(xf.y, -kv));
-                accumulate_dots<NV>(acc, u, x, ml[k]);
-            }
-            w[o] = x;
-        }
-    }
-    if (finish_dots<NV>(acc, s_f, partial, counter, out) && S_slots)
-        for (int o = threadIdx.x; o < kOvSlots * 2 * n * n; o += blockDim.x) S_slots[o] = 0.0;
-}
-
-// Gram-Schmidt update of the raw vector w (the true vector is fw w with
-// fw = s_f[NV-1]): fw w -= sum_{i<NV} c_i q_i, i.e. w -= sum_i (c_i s_f[i] / fw)
-// V_i (interior rows), with the new norm, and the complex64 copy of w in w32
-// when non-null (the input of the next cell pass); the last block writes the
-// Hessenberg column: Hcol[i] = c_i (or += c_i when accumulate),
-// Hcol[NV] = fw |w|_M, and *reorth = 1 when a first pass left
-// |fw w|^2 < eta2 (c[NV] + |fw w|^2), the squared norm before it (c[NV] is
-// its part in the span of the basis).  Skipped when gate && !*gate.
-template <int NV>
-__global__ void __launch_bounds__(kRedThreads) krylov_update_kernel(
-    double2* __restrict__ w, const double2* __restrict__ V, int64_t stride, const double2* __restrict__ c,
-    const double* __restrict__ ml, int64_t n_int, int n, const int* __restrict__ gate, int accumulate, double eta2,
-    int* __restrict__ reorth, const double2* __restrict__ H, int ldh, const double2* __restrict__ beta2,
-    float2* __restrict__ w32, double* __restrict__ partial, unsigned* __restrict__ counter,
-    double2* __restrict__ Hcol) {
-    if (gate && *gate == 0) return;
-    __shared__ double2 s_c[NV + 1];
-    __shared__ double2 s_cf[NV];
-    __shared__ double s_f[NV];
-    krylov_scales(H, ldh, beta2, NV, s_f);
-    if (int(threadIdx.x) <= NV) s_c[threadIdx.x] = c[threadIdx.x];
-    __syncthreads();
-    const double fw = s_f[NV - 1];
-    // the complex64 copy holds 2^kw w with 2^kw ~ fw, i.e. about the true vector
-    // fw w (whose size is the Hessenberg entry): the raw vectors grow like the
-    // operator norm to the power of their index and would leave the binary32
-    // range (project32_dots_kernel undoes the factor)
-    const int kw = fw > 0.0 ? ilogb(fw) : 0;
-    if (int(threadIdx.x) < NV) {
-        const double f = fw > 0.0 ? s_f[threadIdx.x] / fw : 0.0;
-        s_cf[threadIdx.x] = make_double2(s_c[threadIdx.x].x * f, s_c[threadIdx.x].y * f);
-    }
-    __syncthreads();
-    double nrm[1] = {0.0};
-    const RowCol rc(n);
-    if (rc.active) {
-        for (int64_t k = int64_t(blockIdx.x) * rc.R + rc.r; k < n_int; k += int64_t(gridDim.x) * rc.R) {
-            const int64_t o = k * n + rc.p;
-            double2 x = w[o];
-            const double m = ml[k];
-            double2 u[NV];
-#pragma unroll
-            for (int i = 0; i < NV; ++i) u[i] = V[i * stride + o];
-#pragma unroll
-            for (int i = 0; i < NV; ++i) {
-                const double2 h = s_cf[i];
-                x.x = fma(-h.x, u[i].x, fma(h.y, u[i].y, x.x));
-                x.y = fma(-h.x, u[i].y, fma(-h.y, u[i].x, x.y));
-            }
-            w[o] = x;
-            if (w32) w32[o] = make_float2(narrow_f64_scaled(x.x, kw), narrow_f64_scaled(x.y, kw));
-            nrm[0] = fma(m, fma(x.x, x.x, x.y * x.y), nrm[0]);
-        }
-    }
-    block_row_partial<1>(nrm, 1, partial);
-    __shared__ double s_sum[kRedThreads];
-    if (!last_block_sum(partial, 1, counter, s_sum)) return;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < NV; ++i) {
-            const double2 hh = accumulate ? make_double2(Hcol[i].x + s_c[i].x, Hcol[i].y + s_c[i].y) : s_c[i];
-            Hcol[i] = hh;
-        }
-        const double nn = fw * fw * fmax(s_sum[0], 0.0);   // |fw w|^2
-        Hcol[NV] = make_double2(sqrt(nn), 0.0);
-        // |fw w|^2 before the update = in-span part (c[NV]) + what is left (nn)
-        if (reorth) *reorth = (!accumulate && nn < eta2 * (s_c[NV].x + nn)) ? 1 : 0;
-    }
-}
-
-// Closes a substep and opens the next: x = scale sum_{i<M} y_i q_i (q_i =
-// s_f[i] V_i) is written to out (phi after the substep) and, as the next
-// substep's unscaled V_0, to V itself (element by element after its reads),
-// with the complex64 copy in v32 when non-null; the last block writes
-// beta2_out = |x|_M^2 over interior rows.  M = 0 opens the first substep
-// from src (out unused).  beta2_out may be beta2: every block reads beta2 at
-// its start and the last block writes after all others have finished.
-template <int M>
-__global__ void __launch_bounds__(kRedThreads) substep_close_kernel(
-    double2* V, int64_t stride, const double2* __restrict__ y, double scale, const double2* __restrict__ H, int ldh,
-    const double2* beta2, const double2* __restrict__ src, const double* __restrict__ ml, int64_t n_int, int64_t N,
-    int n, double2* __restrict__ out, float2* __restrict__ v32, double* __restrict__ partial,
-    unsigned* __restrict__ counter, double2* beta2_out) {
-    __shared__ double2 s_y[M > 0 ? M : 1];
-    __shared__ double s_f[M > 0 ? M : 1];
-    if (M > 0) krylov_scales(H, ldh, beta2, M, s_f);
-    __syncthreads();
-    if (int(threadIdx.x) < M) {
-        const double f = scale * s_f[threadIdx.x];
-        s_y[threadIdx.x] = make_double2(f * y[threadIdx.x].x, f * y[threadIdx.x].y);
-    }
-    __syncthreads();
-    double nrm[1] = {0.0};
-    const RowCol rc(n);
-    if (rc.active) {
-        for (int64_t k = int64_t(blockIdx.x) * rc.R + rc.r; k < N; k += int64_t(gridDim.x) * rc.R) {
-            const int64_t o = k * n + rc.p;
-            double2 x;
-            if (M == 0) {
-                x = src[o];
             } else {
-                double2 u[M > 0 ? M : 1];
-#pragma unroll
-                for (int i = 0; i < M; ++i) u[i] = V[i * stride + o];
-                x = make_double2(0.0, 0.0);
-#pragma unroll
-                for (int i = 0; i < M; ++i) {
-                    const double2 c = s_y[i];
-                    x.x = fma(c.x, u[i].x, fma(-c.y, u[i].y, x.x));
-                    x.y = fma(c.x, u[i].y, fma(c.y, u[i].x, x.y));
-                }
-                out[o] = x;
+                v = a.S[i];
             }
-            V[o] = x;
-            if (v32) v32[o] = make_float2(narrow_f64(x.x), narrow_f64(x.y));
-            if (k < n_int) nrm[0] = fma(ml[k], fma(x.x, x.x, x.y * x.y), nrm[0]);
+            s_S32[i] = make_float2(narrow_f64(v.x), narrow_f64(v.y));
         }
     }
-    block_row_partial<1>(nrm, 1, partial);
+    if (tid < nv) s_f[tid] = a.f[tid];
+    __syncthreads();
+    // MODE 2: the complex64 input of the cell pass was 2^kv V_{nv-1}
+    // (gs_combine_kernel's scaling; V_0 unscaled), so the raw vector is the
+    // result times 2^-kv
+    const int kv = (MODE == 2 && nv >= 2 && s_f[nv - 2] > 0.0) ? ilogb(s_f[nv - 2]) : 0;
+    const TileRows rc(n);
+    if (rc.active) {
+        const int p = rc.p;
+        BasisStream<E, STAGES> st(a.B, nv, s_v, s_ve);
+#pragma unroll
+        for (int q = 0; q < STAGES - 1; ++q) st.template issue<true>();
+        int slot = 0;
+        const int n_int = int(a.n_int);
+        for (int64_t tile = blockIdx.x; tile < a.B.tiles; tile += gridDim.x) {
+            const int k0 = int(tile) * (E * rc.R) + rc.r;
+            double2 x[E];
+            int kr[E];   // the rows (row 0 in place of those without a part in the sums, whose m w is 0)
+            unsigned xe = 0u;
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                kr[r] = k0 + r * rc.R < n_int ? k0 + r * rc.R : 0;
+                x[r] = make_double2(0.0, 0.0);
+            }
+            if constexpr (MODE == 0) {
+#pragma unroll
+                for (int r = 0; r < E; ++r) {
+                    if (k0 + r * rc.R >= n_int) continue;
+                    const int4 v = a.B.V[nv * a.B.stride + (tile * E + r) * kRedThreads + tid];
+                    const int e = a.B.e[nv * a.B.estride + tile * kRedThreads + tid];
+                    const double sc = e == kFxNan ? __hiloint2double(0x7FF80000, 0) : e == 0 ? 0.0 : ldexp(1.0, e - 1082);
+                    x[r].x = sc * double((static_cast<long long>(v.y) << 32) + v.x);
+                    x[r].y = sc * double((static_cast<long long>(v.w) << 32) + v.z);
+                }
+            }
+            if constexpr (MODE == 1) {
+                double2 zo[E];
+                double s[E];
+#pragma unroll
+                for (int r = 0; r < E; ++r) {
+                    s[r] = a.ml_inv[kr[r]];
+                    zo[r] = a.z[unsigned(kr[r]) * unsigned(n) + unsigned(p)];
+                }
+#pragma unroll
+                for (int r = 0; r < E; ++r) x[r] = make_double2(zo[r].x * s[r], zo[r].y * s[r]);
+                for (int j = 0; j < n; ++j) {
+                    const double2 c = s_S[j * n + p];
+                    double2 f[E];
+#pragma unroll
+                    for (int r = 0; r < E; ++r) f[r] = a.phi[unsigned(kr[r]) * unsigned(n) + unsigned(j)];
+#pragma unroll
+                    for (int r = 0; r < E; ++r) {
+                        x[r].x = fma(-f[r].x, c.x, fma(f[r].y, c.y, x[r].x));
+                        x[r].y = fma(-f[r].x, c.y, fma(-f[r].y, c.x, x[r].y));
+                    }
+                }
+            }
+            if constexpr (MODE == 2) {
+                float2 xf[E];
+                float s[E];
+                const float2* pr[E];
+#pragma unroll
+                for (int r = 0; r < E; ++r) {
+                    s[r] = a.ml_inv32[kr[r]];
+                    xf[r] = a.z32[unsigned(kr[r]) * unsigned(n) + unsigned(p)];
+                    pr[r] = a.phi32 + unsigned(kr[r]) * unsigned(n);
+                }
+                float2 f[4][E];   // four orbitals of the rows in flight
+#pragma unroll
+                for (int j0 = 0; j0 < kMaxOrbProj; j0 += 4) {
+                    if (j0 >= n) break;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int r = 0; r < E; ++r)
+                            if (j0 + j < n) f[j][r] = pr[r][j0 + j];
+                    if (j0 == 0) {
+#pragma unroll
+                        for (int r = 0; r < E; ++r) xf[r] = make_float2(xf[r].x * s[r], xf[r].y * s[r]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (j0 + j < n) {
+                            const float2 c = s_S32[(j0 + j) * n + p];
+#pragma unroll
+                            for (int r = 0; r < E; ++r) {
+                                xf[r].x = fmaf(-f[j][r].x, c.x, fmaf(f[j][r].y, c.y, xf[r].x));
+                                xf[r].y = fmaf(-f[j][r].x, c.y, fmaf(-f[j][r].y, c.x, xf[r].y));
+                            }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < E; ++r) {
+                    x[r] = make_double2(widen_f32_scaled(xf[r].x, -kv), widen_f32_scaled(xf[r].y, -kv));
+                    if (k0 + r * rc.R < n_int) a.z32[unsigned(kr[r]) * unsigned(n) + unsigned(p)] = xf[r];
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                const int k = k0 + r * rc.R;
+                const bool in = k < n_int;
+                if (!in) x[r] = make_double2(0.0, 0.0);
+                if (MODE == 1 && k < int(a.N)) a.wd[unsigned(k) * unsigned(n) + unsigned(p)] = x[r];
+                const double m = in ? a.ml[k] : 0.0;
+                x[r] = make_double2(m * x[r].x, m * x[r].y);
+                xe = max(xe, max(fx_expbits(x[r].x), fx_expbits(x[r].y)));
+            }
+            const int ex = max(int(xe >> 20), kFxMinExp);
+            Fx X[E], Y[E], nX[E];
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                X[r] = fx_make(x[r].x, ex);
+                Y[r] = fx_make(x[r].y, ex);
+                nX[r] = fx_neg(X[r]);
+            }
+            for (int i = 0; i < nv; ++i) {
+                copy_wait<STAGES - 2>();
+                int4 u[E];
+#pragma unroll
+                for (int r = 0; r < E; ++r) u[r] = s_v[(slot * E + r) * kRedThreads + tid];
+                const int eu = s_ve[slot * kRedThreads + tid];
+                slot = slot + 1 == STAGES ? 0 : slot + 1;
+                st.template issue<true>();
+                FxAcc re{0, 0}, im{0, 0};
+#pragma unroll
+                for (int r = 0; r < E; ++r) {
+                    fx_mad(re, fx_re(u[r]), X[r]);
+                    fx_mad(re, fx_im(u[r]), Y[r]);
+                    fx_mad(im, fx_re(u[r]), Y[r]);
+                    fx_mad(im, fx_im(u[r]), nX[r]);
+                }
+                const double sc = fx_scale((eu == kFxNan || xe == kFxExpMask) ? 0x7FFFFF : eu + ex);
+                double2 acc = s_acc[i * kRedThreads + tid];
+                acc.x = fma(fx_value(re), sc, acc.x);
+                acc.y = fma(fx_value(im), sc, acc.y);
+                s_acc[i * kRedThreads + tid] = acc;
+            }
+        }
+    }
+    // block sums: warp j sums the 256 values of vectors j, j + 8, ..
+    __syncthreads();
+    {
+        const int lane = tid & 31, warp = tid >> 5;
+        for (int i = warp; i < nv; i += kRedThreads / 32) {
+            double2 v = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int r = 0; r < kRedThreads / 32; ++r) {
+                const double2 t = s_acc[i * kRedThreads + 32 * r + lane];
+                v.x += t.x;
+                v.y += t.y;
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
+                v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
+            }
+            if (lane == 0) {
+                a.partial[int64_t(blockIdx.x) * 2 * nv + 2 * i] = v.x;
+                a.partial[int64_t(blockIdx.x) * 2 * nv + 2 * i + 1] = v.y;
+            }
+        }
+    }
     __shared__ double s_sum[kRedThreads];
-    if (!last_block_sum(partial, 1, counter, s_sum)) return;
-    if (threadIdx.x == 0) *beta2_out = make_double2(fmax(s_sum[0], 0.0), 0.0);
+    if (!last_block_sum(a.partial, 2 * nv, a.counter, s_sum)) return;
+    const double fw = s_f[nv - 1];
+    if (tid < nv) {
+        const double f = s_f[tid] * fw;
+        a.out[tid] = make_double2(f * s_sum[2 * tid], f * s_sum[2 * tid + 1]);
+    }
+    if (tid == 0) {
+        double nn = 0.0;
+        for (int i = 0; i < nv; ++i) {
+            const double f = s_f[i] * fw;
+            nn += f * f * (s_sum[2 * i] * s_sum[2 * i] + s_sum[2 * i + 1] * s_sum[2 * i + 1]);
+        }
+        a.out[nv] = make_double2(nn, 0.0);
+    }
+    if (MODE == 2 && a.S_slots)
+        for (int o = tid; o < kOvSlots * 2 * n * n; o += blockDim.x) a.S_slots[o] = 0.0;
+}
+
+// Linear combinations of the basis, x = base + sum_{i<nv} c_i V_i, stored as a
+// basis vector with its norm:
+//   KIND 0 opens the first substep: x = src, to V_0;
+//   KIND 1 closes a substep and opens the next: x = scale sum y_i q_i, to out
+//     (phi after the substep; when non-null) and V_0;
+//   KIND 2 is the Gram-Schmidt update of the raw vector w of gs_dots_kernel (the
+//     true vector is fw w with fw = s_f[nv-1]): fw w -= sum c_i q_i, i.e.
+//     w -= sum (c_i s_f[i] / fw) V_i on interior rows (0 on the others), to V_nv;
+//   KIND 4 is the same in the precision form, from the complex64 raw vector;
+//   KIND 3 is the second such pass, on V_nv itself (skipped when !*gate).
+// vd (FP64 form) and v32 (precision form) receive the float64 / complex64 copy
+// of x that the next cell pass reads.  The last block writes beta2_out =
+// |x|_M^2 over interior rows (KIND 0, 1), or the Hessenberg column (KIND 2..4):
+// Hcol[i] = c_i (KIND 3: += c_i), Hcol[nv] = fw |w|_M, and (KIND 2, 4) *reorth = 1
+// when the pass left |fw w|^2 < eta2 (c[nv] + |fw w|^2), the squared norm before
+// it (c[nv] is its part in the span of the basis), and the new scale (every block
+// reads the scales at its start, the last block writes after all others have
+// finished); V_0 is written tile by tile after the tile's reads.
+//
+// A thread brings its group of rows to the scale of the largest term c_i e_i by
+// shifting each coefficient once per group; an element then costs its 16-byte
+// row and 12 IMAD.WIDE per vector, against 4 FP64 multiply-add slots of 64
+// lanes before.  The result keeps 63 bits on the scale of its largest term or
+// of the base and is shifted to the group's new exponent; its squares for the
+// norm are integer products too, rounded to float64 once per row.
+struct GsCombineArgs {
+    KrylovBasis B;
+    int nv;
+    const double2* c;       // KIND 1: y; KIND 2, 3: inner products
+    double scale;           // KIND 1
+    const double2* src;     // KIND 0
+    const double2* wd;      // KIND 2: the raw vector, float64 form
+    const float2* w32;      // KIND 4: the raw vector times 2^kv, precision form
+    const double* ml;
+    int64_t n_int, N;
+    int n;
+    const int* gate;
+    double eta2;
+    int* reorth;
+    double* f;              // the basis's scales
+    double2* out;
+    double2* vd;
+    float2* v32;
+    double* partial;
+    unsigned* counter;
+    double2* Hcol;
+    double2* beta2_out;
+};
+
+// f 2^32 times its own scale over 2^s: the 24-bit significand at bit 32, shifted
+// right by s - e (e the biased exponent of f), with its sign.
+__device__ __forceinline__ long long float_int(float f, int s) {
+    const unsigned u = __float_as_uint(f);
+    const int e = int((u >> 23) & 0xFFu);
+    const unsigned long long m = e == 0 ? 0ull : static_cast<unsigned long long>((u & 0x7FFFFFu) | 0x800000u) << 32;
+    const unsigned long long v = m >> min(s - e, 63);
+    return int(u) < 0 ? -static_cast<long long>(v) : static_cast<long long>(v);
+}
+
+constexpr int kCombineStages = 4;
+template <int E, int KIND>
+__global__ void __launch_bounds__(kRedThreads, 2) gs_combine_kernel(const __grid_constant__ GsCombineArgs a) {
+    if (KIND == 3 && *a.gate == 0) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int4* s_v = reinterpret_cast<int4*>(smem_raw);                                   // [stages][E][kRedThreads]
+    int* s_ge = reinterpret_cast<int*>(s_v + kCombineStages * E * kRedThreads);     // [2][nv][kRedThreads]
+    __shared__ double s_f[kMaxKrylov];
+    __shared__ double2 s_c[kMaxKrylov + 1];
+    __shared__ longlong2 s_ci[kMaxKrylov];   // coefficients, integers on their own scale
+    __shared__ int s_ce[kMaxKrylov];         // their biased exponents
+    __shared__ int s_low;                    // smallest admissible term exponent (kFxMaxSum + 1: NaN)
+    const int nv = a.nv, n = a.n, tid = threadIdx.x;
+    double fw = 1.0;
+    int kw = 0, kv = 0;
+    if constexpr (KIND != 0) {
+        if (tid < nv) s_f[tid] = a.f[tid];
+        if (tid <= (KIND == 1 ? nv - 1 : nv)) s_c[tid] = a.c[tid];
+        __syncthreads();
+        if constexpr (KIND >= 2) {
+            fw = s_f[nv - 1];
+            // the complex64 copy holds 2^kw w with 2^kw ~ fw, i.e. about the true
+            // vector fw w (whose size is the Hessenberg entry): the raw vectors
+            // grow like the operator norm to the power of their index and would
+            // leave the binary32 range (gs_dots_kernel undoes the factor)
+            kw = fw > 0.0 ? ilogb(fw) : 0;
+            if (nv >= 2 && s_f[nv - 2] > 0.0) kv = ilogb(s_f[nv - 2]);   // the cell pass's factor 2^kv in w32
+        }
+        if (tid < nv) {
+            const double f = KIND == 1 ? a.scale * s_f[tid] : fw > 0.0 ? -s_f[tid] / fw : 0.0;
+            const double2 c = make_double2(f * s_c[tid].x, f * s_c[tid].y);
+            const int e = int(max(fx_expbits(c.x), fx_expbits(c.y)) >> 20);
+            s_ce[tid] = e;
+            s_ci[tid] = make_longlong2(e ? fx_int(c.x, e) : 0, e ? fx_int(c.y, e) : 0);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            int m = 1023;
+            bool bad = false;
+            for (int i = 0; i < nv; ++i) {
+                m = max(m, s_ce[i]);
+                bad = bad || s_ce[i] == 0x7FF;
+            }
+            s_low = bad ? kFxMaxSum + 1 : m + kFxMinExp;
+        }
+        __syncthreads();
+    }
+    const TileRows rc(n);
+    const int p = rc.p;
+    double nrm[1] = {0.0};
+    // the group exponents of this and the next tile, staged like the vectors
+    auto copy_e = [&](int64_t tile, int par) {
+        if (tile < a.B.tiles)
+            for (int i = 0; i < nv; ++i)
+                copy4(s_ge + (par * nv + i) * kRedThreads + tid, a.B.e + i * a.B.estride + tile * kRedThreads + tid);
+    };
+    BasisStream<E, kCombineStages> st(a.B, nv, s_v, s_ge);
+    if (KIND != 0 && rc.active) {
+        copy_e(blockIdx.x, 0);   // complete with the first item
+#pragma unroll
+        for (int q = 0; q < kCombineStages - 1; ++q) st.template issue<false>();
+    }
+    int slot = 0, par = 0;
+    const int N = int(a.N), n_int = int(a.n_int);
+    const int rows = KIND >= 2 ? n_int : N;   // rows of the result; zero beyond
+    for (int64_t tile = blockIdx.x; rc.active && tile < a.B.tiles; tile += gridDim.x, par ^= 1) {
+        int* eg = a.B.e + tile * kRedThreads + tid;
+        const int k0 = int(tile) * (E * rc.R) + rc.r;
+        unsigned o[E];
+        long long tx[E], ty[E];
+        float2 bf[E];    // the base and the masses: loaded ahead of the walk
+        double mass[E];
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int k = k0 + r * rc.R;
+            o[r] = unsigned(k < N ? k : 0) * unsigned(n) + unsigned(p);
+            tx[r] = ty[r] = 0;
+            mass[r] = k < n_int ? a.ml[k] : 0.0;
+            bf[r] = make_float2(0.f, 0.f);
+            if (KIND == 4 && k < n_int) bf[r] = a.w32[o[r]];
+        }
+        int EM = KIND == 0 ? 1023 + kFxMinExp : s_low;
+        if constexpr (KIND != 0) {
+            // this tile's exponents came with an item at least nv before its own
+            if (tile == blockIdx.x) copy_wait<kCombineStages - 2>();
+            else if (nv < kCombineStages) copy_wait<0>();
+            const int* ge = s_ge + par * nv * kRedThreads + tid;
+            bool bad = false;
+#pragma unroll 4
+            for (int i = 0; i < nv; ++i) {
+                const int e = ge[i * kRedThreads];
+                bad = bad || e == kFxNan;
+                EM = max(EM, e + s_ce[i]);
+            }
+            copy_e(tile + gridDim.x, par ^ 1);   // in the next item's group
+            FxAcc ax[E], ay[E];
+#pragma unroll
+            for (int r = 0; r < E; ++r) ax[r] = ay[r] = FxAcc{0, 0};
+            for (int i = 0; i < nv; ++i) {
+                const int sh = min(EM - ge[i * kRedThreads] - s_ce[i], 63);
+                const longlong2 ci = s_ci[i];
+                const Fx re = fx_split(ci.x >> sh), im = fx_split(ci.y >> sh), nim = fx_split(-(ci.y >> sh));
+                copy_wait<kCombineStages - 2>();
+                int4 u[E];
+#pragma unroll
+                for (int r = 0; r < E; ++r) u[r] = s_v[(slot * E + r) * kRedThreads + tid];
+                slot = slot + 1 == kCombineStages ? 0 : slot + 1;
+                st.template issue<false>();
+#pragma unroll
+                for (int r = 0; r < E; ++r) {
+                    fx_mad(ax[r], re, fx_re(u[r]));
+                    fx_mad(ax[r], nim, fx_im(u[r]));
+                    fx_mad(ay[r], re, fx_im(u[r]));
+                    fx_mad(ay[r], im, fx_re(u[r]));
+                }
+                if (i & 1) {   // two vectors (4 products) between carries
+#pragma unroll
+                    for (int r = 0; r < E; ++r) {
+                        fx_carry(ax[r]);
+                        fx_carry(ay[r]);
+                    }
+                }
+            }
+            if (bad) EM = kFxMaxSum + 1;
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                tx[r] = (ax[r].hh << 1) + (ax[r].x >> 31);
+                ty[r] = (ay[r].hh << 1) + (ay[r].x >> 31);
+            }
+        }
+        if constexpr (KIND == 4) {   // the base: 24 bits at 2^56 of the scale EM, the thread's rows alike
+            unsigned be = 0u;
+#pragma unroll
+            for (int r = 0; r < E; ++r)
+                be = max(be, max(__float_as_uint(bf[r].x) & 0x7F800000u, __float_as_uint(bf[r].y) & 0x7F800000u));
+            const int eb = max(int(be >> 23) + 896 - kv, kFxMinExp);
+            const int up = max(EM, eb + 1023), d = min(up - EM, 63);
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                tx[r] = (tx[r] >> d) + float_int(bf[r].x, up - 1919 + kv);
+                ty[r] = (ty[r] >> d) + float_int(bf[r].y, up - 1919 + kv);
+            }
+            EM = (EM > kFxMaxSum || be == 0x7F800000u || eb >= kFxNan) ? kFxMaxSum + 1 : up;
+        } else if constexpr (KIND != 1) {   // the base: 53 bits at 2^56 of the scale EM
+            double2 b[E];
+            unsigned be = 0u;
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                const int k = k0 + r * rc.R;
+                b[r] = make_double2(0.0, 0.0);
+                if (k < rows) {
+                    if constexpr (KIND == 0) b[r] = a.src[o[r]];
+                    if constexpr (KIND == 2) b[r] = a.wd[o[r]];
+                    if constexpr (KIND == 3) {
+                        const int4 v = a.B.V[nv * a.B.stride + (tile * E + r) * kRedThreads + tid];
+                        const int e = eg[nv * a.B.estride];
+                        const double sc = e == kFxNan ? __hiloint2double(0x7FF80000, 0)
+                                                      : e == 0 ? 0.0 : ldexp(1.0, e - 1082);
+                        b[r].x = sc * double((static_cast<long long>(v.y) << 32) + v.x);
+                        b[r].y = sc * double((static_cast<long long>(v.w) << 32) + v.z);
+                    }
+                }
+                be = max(be, max(fx_expbits(b[r].x), fx_expbits(b[r].y)));
+            }
+            const int eb = max(int(be >> 20), kFxMinExp);
+            const int up = max(EM, eb + 1023), d = min(up - EM, 63);
+            const int es = min(up - 1023, 8000);   // b 2^(2101 - up) = (b 2^(1082 - es)) / 16 for es = up - 1023
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                tx[r] = (tx[r] >> d) + (fx_int(b[r].x, es) >> 4);
+                ty[r] = (ty[r] >> d) + (fx_int(b[r].y, es) >> 4);
+            }
+            EM = (EM > kFxMaxSum || be == kFxExpMask) ? kFxMaxSum + 1 : up;
+        }
+        unsigned long long any = 0ull;
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            if (k0 + r * rc.R >= rows) tx[r] = ty[r] = 0;
+            any |= static_cast<unsigned long long>((tx[r] ^ (tx[r] >> 63)) | (ty[r] ^ (ty[r] >> 63)));
+        }
+        const int bits = 64 - __clzll(static_cast<long long>(any));
+        // the group's new exponent: |x| <= 2^(bits + EM - 2101) (t = -1 alone: any = 0)
+        int eo = bits ? bits + EM - 1079 : 0;
+        if (EM > kFxMaxSum || eo > kFxNan) eo = kFxNan;
+        if (eo < kFxMinExp) eo = 0;
+        const int dst = KIND <= 1 ? 0 : nv;
+        eg[dst * a.B.estride] = eo;
+        const int shl = 63 - bits;   // t 2^(EM - 2101) = X 2^(eo - 1082), X = t 2^(60 - bits)
+        double n2 = 0.0;
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int k = k0 + r * rc.R;
+            if (k >= N) continue;
+            long long vx = 0, vy = 0;
+            if (eo != 0) {
+                vx = (tx[r] << shl) >> 3;
+                vy = (ty[r] << shl) >> 3;
+            }
+            const Fx fx = fx_split(vx), fy = fx_split(vy);
+            a.B.V[dst * a.B.stride + (tile * E + r) * kRedThreads + tid] = make_int4(fx.l, fx.h, fy.l, fy.h);
+            FxAcc sq{0, 0};
+            fx_mad(sq, fx, fx);
+            fx_mad(sq, fy, fy);
+            n2 = fma(mass[r], fx_value(sq), n2);
+            if ((KIND == 1 && a.out) || a.vd) {
+                const double sc = fx_scale(EM);
+                const double2 v = make_double2(__ll2double_rn(tx[r]) * sc, __ll2double_rn(ty[r]) * sc);
+                if (KIND == 1 && a.out) a.out[o[r]] = v;
+                if (a.vd) a.vd[o[r]] = v;
+            }
+            if (a.v32) a.v32[o[r]] = make_float2(fx_to_f32(vx, eo - 1082 + kw), fx_to_f32(vy, eo - 1082 + kw));
+        }
+        nrm[0] = fma(n2, eo == kFxNan ? __hiloint2double(0x7FF80000, 0) : fx_scale(2 * eo), nrm[0]);
+    }
+    __syncthreads();
+    block_row_partial<1>(nrm, 1, a.partial);
+    __shared__ double s_sum[kRedThreads];
+    if (!last_block_sum(a.partial, 1, a.counter, s_sum)) return;
+    if (tid == 0) {
+        if constexpr (KIND <= 1) {
+            const double b2 = fmax(s_sum[0], 0.0), beta = sqrt(b2);
+            *a.beta2_out = make_double2(b2, 0.0);
+            a.f[0] = beta > 0.0 ? 1.0 / beta : 0.0;
+            a.f[kScaleBeta] = beta;
+        } else {
+            for (int i = 0; i < nv; ++i) {
+                const double2 h = KIND == 3 ? make_double2(a.Hcol[i].x + s_c[i].x, a.Hcol[i].y + s_c[i].y) : s_c[i];
+                a.Hcol[i] = h;
+            }
+            const double nn = fw * fw * fmax(s_sum[0], 0.0);   // |fw w|^2
+            const double h = sqrt(nn);
+            a.Hcol[nv] = make_double2(h, 0.0);
+            a.f[nv] = (h > 1e-14 * a.f[kScaleBeta] && h > 0.0) ? fw / h : 0.0;
+            // |fw w|^2 before the update = in-span part (c[nv]) + what is left (nn)
+            if (KIND != 3) *a.reorth = nn < a.eta2 * (s_c[nv].x + nn) ? 1 : 0;
+        }
+    }
 }
 
 // exp(-i dt H) (imag: exp(-dt H), the imaginary-time step) for an m x m
@@ -769,131 +1086,68 @@ int to_c64(const double2* x, float2* y, int64_t n, cudaStream_t s) {
 int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const float2* U, float2* z, int n,
                     cudaStream_t s, int velocity, const float2* U_hang = nullptr);
 
-#define AFEM_NV_CASES(X) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16)
-
-// One resident wave of kernel K (its occupancy per SM x the SMs), at most
-// `cap` blocks: the FP64-bound Gram-Schmidt kernels then have no tail wave,
-// and each thread covers more rows per FP64 block reduction.
+// Blocks of kernel K for `tiles` tiles: one resident wave at most (every block
+// then takes several tiles and adds one row of partial sums).
 template <auto K>
-static unsigned wave_grid(unsigned cap) {
-    static const int per_sm = [] {
+static unsigned wave_grid(int64_t tiles, size_t smem) {
+    static const int per_sm = [smem] {
         int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, K, kRedThreads, 0) != cudaSuccess || b < 1) b = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, K, kRedThreads, smem) != cudaSuccess || b < 1) b = 1;
         return b;
     }();
-    const unsigned g = unsigned(device_sms() * per_sm);
-    return g < cap ? g : cap;
+    const int64_t cap = std::min<int64_t>(int64_t(device_sms()) * per_sm, red_blocks());
+    return unsigned(std::max<int64_t>(1, std::min(tiles, cap)));
 }
 
-// The Gram-Schmidt kernels for a run-time vector count nv (0 <= nv <= kMaxKrylov).
-static int launch_krylov_dots(int nv, unsigned grid, cudaStream_t s, const double2* w, const double2* V,
-                              int64_t stride, const double* ml, int64_t n_int, int n, const int* gate,
-                              const double2* H, int ldh, const double2* beta2, double* partial, unsigned* counter,
-                              double2* out) {
-    switch (nv) {
-        case 0:
-            AFEM_LAUNCH((krylov_dots_kernel<0>), wave_grid<krylov_dots_kernel<0>>(grid), kRedThreads, 0, s, w, V,
-                        stride, ml, n_int, n, gate, H, ldh,
-                        beta2, partial, counter, out);
-            break;
-#define AFEM_DOTS_CASE(NVV)                                                                                       \
-    case NVV:                                                                                                     \
-        AFEM_LAUNCH((krylov_dots_kernel<NVV>), wave_grid<krylov_dots_kernel<NVV>>(grid), kRedThreads, 0, s, w, V, \
-                    stride, ml, n_int, n, gate, H, ldh,                                                       \
-                    beta2, partial, counter, out);                                                                \
-        break;
-            AFEM_NV_CASES(AFEM_DOTS_CASE)
-#undef AFEM_DOTS_CASE
-        default:
-            return set_error(AFEM_EINVAL, "arnoldi: Krylov vector count out of range");
-    }
-    AFEM_CUDA_TRY(cudaGetLastError());
-    return AFEM_OK;
-}
-
-// The projector of G on the cell-pass output fused with the inner products
-// against V_0..V_{nv-1}: complex64 z (precision form, phi32) or complex128 z.
-static int launch_project_dots(int nv, unsigned grid, cudaStream_t s, const float2* z32, const float2* phi32,
-                               const double2* z, const double2* phi, const double2* S, const DeviceMesh& D, int n,
-                               double2* w, const double2* V, int64_t stride, const double2* H, int ldh,
-                               const double2* beta2, double* partial, unsigned* counter, double2* out,
-                               double* S_slots) {
-    switch (nv) {
-#define AFEM_PD_CASE(NVV)                                                                                           \
-    case NVV:                                                                                                       \
-        if (z32) {                                                                                                  \
-            AFEM_LAUNCH((project32_dots_kernel<NVV>), wave_grid<project32_dots_kernel<NVV>>(grid), kRedThreads, 0, \
-                        s, z32, phi32, S, D.ml_inv32, D.ml,                                                         \
-                        D.n_interior, D.n_master, n, w, V, stride, H, ldh, beta2, partial, counter, out, S_slots);  \
-        } else {                                                                                                    \
-            AFEM_LAUNCH((project_dots_kernel<NVV>), wave_grid<project_dots_kernel<NVV>>(grid), kRedThreads, 0, s, \
-                        z, phi, S, D.ml_inv, D.ml,                                                                  \
-                        D.n_interior, D.n_master, n, w, V, stride, H, ldh, beta2, partial, counter, out);           \
-        }                                                                                                           \
-        break;
-        AFEM_NV_CASES(AFEM_PD_CASE)
-#undef AFEM_PD_CASE
-        default:
-            return set_error(AFEM_EINVAL, "arnoldi: Krylov vector count out of range");
-    }
-    AFEM_CUDA_TRY(cudaGetLastError());
-    return AFEM_OK;
-}
-
-static int launch_krylov_update(int nv, unsigned grid, cudaStream_t s, double2* w, const double2* V,
-                                int64_t stride, const double2* c, const double* ml, int64_t n_int, int n,
-                                const int* gate, int accumulate, double eta2, int* reorth, const double2* H, int ldh,
-                                const double2* beta2, float2* w32, double* partial, unsigned* counter,
-                                double2* Hcol) {
-    switch (nv) {
-#define AFEM_UPD_CASE(NVV)                                                                                      \
-    case NVV:                                                                                                   \
-        AFEM_LAUNCH((krylov_update_kernel<NVV>), wave_grid<krylov_update_kernel<NVV>>(grid), kRedThreads, 0, s, \
-                    w, V, stride, c, ml, n_int, n, gate,                                                          \
-                    accumulate, eta2, reorth, H, ldh, beta2, w32, partial, counter, Hcol);                      \
-        break;
-        AFEM_NV_CASES(AFEM_UPD_CASE)
-#undef AFEM_UPD_CASE
-        default:
-            return set_error(AFEM_EINVAL, "arnoldi: Krylov vector count out of range");
-    }
-    AFEM_CUDA_TRY(cudaGetLastError());
-    return AFEM_OK;
-}
-
-// substep_close_kernel for m = 0 (open the first substep from src) or the
-// substep's Krylov dimension m (1..kMaxKrylov).
-static int launch_substep_close(int m, unsigned grid, cudaStream_t s, double2* V, int64_t stride, const double2* y,
-                                double scale, const double2* H, int ldh, double2* beta2, const double2* src,
-                                const DeviceMesh& D, int n, double2* out, float2* v32, double* partial,
-                                unsigned* counter) {
-    switch (m) {
-        case 0:
-            AFEM_LAUNCH((substep_close_kernel<0>), wave_grid<substep_close_kernel<0>>(grid), kRedThreads, 0, s, V,
-                        stride, y, scale, H, ldh, beta2, src, D.ml, D.n_interior, D.n_master, n, out, v32, partial,
-                        counter, beta2);
-            break;
-#define AFEM_CLOSE_CASE(MM)                                                                                   \
-    case MM:                                                                                                  \
-        AFEM_LAUNCH((substep_close_kernel<MM>), wave_grid<substep_close_kernel<MM>>(grid), kRedThreads, 0, s, \
-                    V, stride, y, scale, H, ldh, beta2, src, D.ml, D.n_interior, D.n_master, n, out, v32,      \
-                    partial, counter, beta2);                                                                 \
-        break;
-            AFEM_NV_CASES(AFEM_CLOSE_CASE)
-#undef AFEM_CLOSE_CASE
-        default:
-            return set_error(AFEM_EINVAL, "arnoldi: Krylov dimension out of range");
-    }
-    AFEM_CUDA_TRY(cudaGetLastError());
-    return AFEM_OK;
-}
-
-static unsigned rowcol_grid(int64_t rows, int n) {
+// Rows of a tile per thread: as many as leave the chip several tiles per SM
+// (4: two float64 additions per vector serve four rows; 1 on small meshes,
+// where blocks in flight count for more).
+static int krylov_rows(int64_t N, int n) {
     const int64_t R = kRedThreads / n;
-    int64_t g = (rows + R - 1) / R;
-    if (g < 1) g = 1;
-    if (g > red_blocks()) g = red_blocks();
-    return unsigned(g);
+    for (int E = 4; E > 1; E >>= 1)
+        if ((N + E * R - 1) / (E * R) >= 4 * device_sms()) return E;
+    return 1;
+}
+
+// STAGES: as many as leave two blocks per SM beside the sums of nv vectors.
+template <int E, int MODE, int STAGES>
+static int launch_gs_dots_s(const GsDotsArgs& a, cudaStream_t s) {
+    constexpr size_t kStage = size_t(STAGES) * kRedThreads * (E * sizeof(int4) + sizeof(int));
+    AFEM_CUDA_TRY(allow_dyn_smem(gs_dots_kernel<E, MODE, STAGES>));
+    const unsigned g = wave_grid<gs_dots_kernel<E, MODE, STAGES>>(
+        a.B.tiles, (STAGES == 4 ? 10 : STAGES == 3 ? 14 : 16) * kRedThreads * sizeof(double2) + kStage);
+    AFEM_LAUNCH((gs_dots_kernel<E, MODE, STAGES>), g, kRedThreads, a.nv * kRedThreads * sizeof(double2) + kStage, s, a);
+    AFEM_CUDA_TRY(cudaGetLastError());
+    return AFEM_OK;
+}
+template <int E, int MODE>
+static int launch_gs_dots_e(const GsDotsArgs& a, cudaStream_t s) {
+    return a.nv <= 10 ? launch_gs_dots_s<E, MODE, 4>(a, s) : a.nv <= 14 ? launch_gs_dots_s<E, MODE, 3>(a, s)
+                                                                        : launch_gs_dots_s<E, MODE, 2>(a, s);
+}
+template <int MODE>
+static int launch_gs_dots(int E, const GsDotsArgs& a, cudaStream_t s) {
+    if (a.nv < 1 || a.nv > kMaxKrylov) return set_error(AFEM_EINVAL, "arnoldi: Krylov vector count out of range");
+    return E == 4 ? launch_gs_dots_e<4, MODE>(a, s) : E == 2 ? launch_gs_dots_e<2, MODE>(a, s)
+                                                            : launch_gs_dots_e<1, MODE>(a, s);
+}
+
+template <int E, int KIND>
+static int launch_gs_combine_e(const GsCombineArgs& a, cudaStream_t s) {
+    constexpr size_t kStage = KIND == 0 ? 0 : size_t(kCombineStages) * kRedThreads * E * sizeof(int4);
+    constexpr size_t kExp = KIND == 0 ? 0 : 2 * kRedThreads * sizeof(int);   // per vector
+    AFEM_CUDA_TRY(allow_dyn_smem(gs_combine_kernel<E, KIND>));
+    const unsigned g = wave_grid<gs_combine_kernel<E, KIND>>(a.B.tiles, kStage + kMaxKrylov * kExp);
+    AFEM_LAUNCH((gs_combine_kernel<E, KIND>), g, kRedThreads, kStage + a.nv * kExp, s, a);
+    AFEM_CUDA_TRY(cudaGetLastError());
+    return AFEM_OK;
+}
+template <int KIND>
+static int launch_gs_combine(int E, const GsCombineArgs& a, cudaStream_t s) {
+    if (a.nv < (KIND == 0 ? 0 : 1) || a.nv > kMaxKrylov)
+        return set_error(AFEM_EINVAL, "arnoldi: Krylov vector count out of range");
+    return E == 4 ? launch_gs_combine_e<4, KIND>(a, s) : E == 2 ? launch_gs_combine_e<2, KIND>(a, s)
+                                                               : launch_gs_combine_e<1, KIND>(a, s);
 }
 
 // The cell pass of G and the projector overlaps S[j][p] = phi_j^H z_p (equal to
@@ -948,8 +1202,15 @@ static int g_cell_overlaps(afem_mesh* m, const double* E, const double2* phi, co
 
 int arnoldi_reserve(afem_mesh* m, int n, int mk, ArnoldiWork& w) {
     const size_t NV = size_t(m->dev.n_master) * n;
+    w.rows = krylov_rows(m->dev.n_master, n);
+    const int64_t tile = int64_t(w.rows) * (kRedThreads / n);
+    w.B.tiles = (m->dev.n_master + tile - 1) / tile;
+    w.B.stride = w.B.tiles * w.rows * kRedThreads;
+    w.B.estride = w.B.tiles * kRedThreads;
     auto carve = [&](Carver& cv) {
-        w.V = cv.take<double2>(size_t(mk + 1) * NV);
+        w.B.V = cv.take<int4>(size_t(mk + 1) * w.B.stride);
+        w.B.e = cv.take<int>(size_t(mk + 1) * w.B.estride);
+        w.vd = cv.take<double2>(NV);
         w.z = cv.take<double2>(NV);
         w.cpartial = cv.take<double2>(size_t(kRedBlocksMax) * 256);
         w.S = cv.take<double2>(kMaxOrbProj * kMaxOrbProj);
@@ -957,6 +1218,7 @@ int arnoldi_reserve(afem_mesh* m, int n, int mk, ArnoldiWork& w) {
         w.res = cv.take<double2>(kResSize);
         w.c1 = cv.take<double2>(kMaxKrylov + 1);
         w.c2 = cv.take<double2>(kMaxKrylov + 1);
+        w.f = cv.take<double>(kScaleBeta + 1);
         w.v32 = cv.take<float2>(NV);
         w.z32 = cv.take<float2>(NV);
         w.phi32 = cv.take<float2>(NV);
@@ -973,7 +1235,6 @@ int arnoldi_reserve(afem_mesh* m, int n, int mk, ArnoldiWork& w) {
     if (rc) return rc;
     Carver cv(m->ws_arnoldi.ptr);
     carve(cv);
-    w.stride = int64_t(NV);
     w.H = w.res + kResH;
     w.beta2 = w.res + kResBeta2;
     w.col = w.res + kResCol;
@@ -1015,7 +1276,7 @@ int arnoldi_step(afem_mesh* m, const double* E, const double2* phi, const double
     ArnoldiWork w{};
     int rc = arnoldi_reserve(m, n, mk, w);
     if (rc) return rc;
-    const int64_t NV = w.stride;
+    const int64_t NV = D.n_master * n;
     const bool projector = !(flags & kArnNoProjector);
     // candidate exponentials exp(-i tau H_m), or exp(+i tau H_m) propagating backward
     auto signed_ladder = [&](double tm, int K) {
@@ -1062,8 +1323,6 @@ int arnoldi_step(afem_mesh* m, const double* E, const double2* phi, const double
     AFEM_CUDA_TRY(cudaMemsetAsync(w.flag, 0, 4 * sizeof(int), s));
     AFEM_CUDA_TRY(cudaMemsetAsync(w.Sslots, 0, sizeof(double) * kOvSlots * 2 * kMaxOrbProj * kMaxOrbProj, s));
     const int ldh = kMaxKrylov + 1;
-    const unsigned gdots = rowcol_grid(D.n_interior, n);
-    const unsigned gproj = rowcol_grid(D.n_master, n);
     double* part = reinterpret_cast<double*>(w.cpartial);
     unsigned* cnt = w.counters + 1;
     const double eta2 = 1e-4;   // second pass when the update left less than 1e-2 of the norm
@@ -1078,17 +1337,58 @@ int arnoldi_step(afem_mesh* m, const double* E, const double2* phi, const double
             return set_error(AFEM_ECUDA, "arnoldi: a G cell pass gave up waiting for a per-cell block copy");
         return AFEM_OK;
     };
-    float2* v32 = mixed ? w.v32 : nullptr;
-    // V_0 = phi (unscaled), its complex64 copy and beta^2 = <phi, phi>_M; later
-    // substeps get theirs from the closing pass of the previous one
-    if ((rc = launch_substep_close(0, gproj, s, w.V, NV, nullptr, 0.0, w.H, ldh, w.beta2, phi, D, n, nullptr, v32,
-                                   part, cnt)))
-        return rc;
+    GsDotsArgs da{};
+    da.z = w.z;
+    da.z32 = w.z32;
+    da.phi = phi;
+    da.phi32 = w.phi32;
+    da.S = w.S;
+    da.S_slots = (mixed && projector) ? w.Sslots : nullptr;
+    da.ml_inv = D.ml_inv;
+    da.ml_inv32 = D.ml_inv32;
+    da.ml = D.ml;
+    da.n_int = D.n_interior;
+    da.N = D.n_master;
+    da.n = n;
+    da.wd = w.vd;
+    da.B = w.B;
+    da.f = w.f;
+    da.partial = part;
+    da.counter = cnt;
+    GsCombineArgs ca{};
+    ca.B = w.B;
+    ca.src = phi;
+    ca.wd = w.vd;
+    ca.w32 = mixed ? w.z32 : nullptr;
+    ca.ml = D.ml;
+    ca.n_int = D.n_interior;
+    ca.N = D.n_master;
+    ca.n = n;
+    ca.gate = w.flag;
+    ca.eta2 = eta2;
+    ca.reorth = w.flag;
+    ca.f = w.f;
+    ca.vd = mixed ? nullptr : w.vd;
+    ca.v32 = mixed ? w.v32 : nullptr;
+    ca.partial = part;
+    ca.counter = cnt;
+    ca.beta2_out = w.beta2;
+    // V_0 = phi (unscaled), the cell pass's copy of it and beta^2 = <phi, phi>_M;
+    // later substeps get theirs from the closing pass of the previous one
+    if ((rc = launch_gs_combine<0>(w.rows, ca, s))) return rc;
+    // closes a substep with the coefficients y = beta exp(..) e_1; phi_out is
+    // written by the last one alone
+    auto close = [&](int mu, const double2* y, double beta, bool last) -> int {
+        ca.nv = mu;
+        ca.c = y;
+        ca.scale = beta;
+        ca.out = last ? phi_out : nullptr;
+        return launch_gs_combine<1>(w.rows, ca, s);
+    };
     while (remaining > 0.0) {
         if (substeps >= 4096) return set_error(AFEM_EINVAL, "arnoldi: more than 4096 substeps (tolerance too tight)");
         AFEM_CUDA_TRY(cudaMemsetAsync(w.H, 0, sizeof(double2) * ldh * kMaxKrylov, s));
         for (int j = 0; j < mk; ++j) {
-            double2* Wn = w.V + (j + 1) * NV;
             double2* Hcol = w.H + j * ldh;
             // w = G q_j (the cell pass on the stored V_j, scaled in the projector
             // pass) with the inner products against q_0..q_j, the update (which
@@ -1100,33 +1400,34 @@ int arnoldi_step(afem_mesh* m, const double* E, const double2* phi, const double
                               : launch_g_cell32(m, E, w.v32, U32, w.z32, n, s, velocity, w.uh32);
                     if (rc) return rc;
                 } else {
-                    if ((rc = launch_g_cell(m, E, w.V + j * NV, U, w.z, n, s, velocity, w.uh))) return rc;
+                    if ((rc = launch_g_cell(m, E, w.vd, U, w.z, n, s, velocity, w.uh))) return rc;
                 }
             } else if (mixed) {
                 if ((rc = g_cell_overlaps32(m, E, w.phi32, U32, n, w.v32, w, s, velocity))) return rc;
             } else {
-                if ((rc = g_cell_overlaps(m, E, phi, U, n, w.V + j * NV, w, s, velocity))) return rc;
+                if ((rc = g_cell_overlaps(m, E, phi, U, n, w.vd, w, s, velocity))) return rc;
             }
             // algorithmic FP64 flops per element: 8 per basis vector in each pass
             // (one complex multiply-add), plus 4 for the new norm in the update
             const double gs_flops = double(D.n_interior) * n * 8.0 * (j + 1);
             {
                 ProfScope ps(AFEM_PROF_GS, s, gs_flops);
-                rc = launch_project_dots(j + 1, gproj, s, mixed ? w.z32 : nullptr, w.phi32, w.z, phi, w.S, D, n, Wn,
-                                         w.V, NV, w.H, ldh, w.beta2, part, cnt, w.c1,
-                                         (mixed && projector) ? w.Sslots : nullptr);
+                da.nv = j + 1;
+                da.gate = nullptr;
+                da.out = w.c1;
+                rc = mixed ? launch_gs_dots<2>(w.rows, da, s) : launch_gs_dots<1>(w.rows, da, s);
             }
+            ca.nv = j + 1;
+            ca.c = w.c1;
+            ca.Hcol = Hcol;
             if (!rc) {
                 ProfScope ps(AFEM_PROF_GS, s, gs_flops + double(D.n_interior) * n * 4.0);
-                rc = launch_krylov_update(j + 1, gdots, s, Wn, w.V, NV, w.c1, D.ml, D.n_interior, n, nullptr, 0, eta2,
-                                          w.flag, w.H, ldh, w.beta2, v32, part, cnt, Hcol);
+                rc = mixed ? launch_gs_combine<4>(w.rows, ca, s) : launch_gs_combine<2>(w.rows, ca, s);
             }
-            if (rc ||
-                (rc = launch_krylov_dots(j + 1, gdots, s, Wn, w.V, NV, D.ml, D.n_interior, n, w.flag, w.H, ldh,
-                                         w.beta2, part, cnt, w.c2)) ||
-                (rc = launch_krylov_update(j + 1, gdots, s, Wn, w.V, NV, w.c2, D.ml, D.n_interior, n, w.flag, 1,
-                                           eta2, nullptr, w.H, ldh, w.beta2, v32, part, cnt, Hcol)))
-                return rc;
+            da.gate = w.flag;
+            da.out = w.c2;
+            ca.c = w.c2;
+            if (rc || (rc = launch_gs_dots<0>(w.rows, da, s)) || (rc = launch_gs_combine<3>(w.rows, ca, s))) return rc;
             if (adaptive) {
                 // Sec. 3.2's rule: the estimate of dimension j + 1 at the fixed step;
                 // the first dimension that meets the threshold (or breaks down) ends
@@ -1151,9 +1452,7 @@ int arnoldi_step(afem_mesh* m, const double* E, const double2* phi, const double
             tau = tau_fixed;
             err = brk ? 0.0 : beta * res[kResErr].x;
             if (!brk && res[kResErr].x > tol) ++unmet;
-            if ((rc = launch_substep_close(m_used, gproj, s, w.V, NV, w.col, beta, w.H, ldh, w.beta2, nullptr, D, n,
-                                           phi_out, v32, part, cnt)))
-                return rc;
+            if ((rc = close(m_used, w.col, beta, substeps + 1 >= adaptive_steps || !(remaining - tau > 0.0)))) return rc;
             err_sum += err;
             ++substeps;
             dim_max = std::max(dim_max, m_used);
@@ -1214,8 +1513,7 @@ int arnoldi_step(afem_mesh* m, const double* E, const double2* phi, const double
         tau = make_ladder(tau_max, K).tau[pick];
         err = beta * res[kResErr + pick].x;
         // phi_out = beta V_m exp(-i tau H_m) e_1, which also opens the next substep
-        if ((rc = launch_substep_close(m_used, gproj, s, w.V, NV, w.col + pick * kMaxKrylov, beta, w.H, ldh, w.beta2,
-                                       nullptr, D, n, phi_out, v32, part, cnt)))
+        if ((rc = close(m_used, w.col + pick * kMaxKrylov, beta, tau >= remaining || !(remaining - tau > 0.0))))
             return rc;
         err_sum += err;
         ++substeps;

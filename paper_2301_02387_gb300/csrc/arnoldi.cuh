@@ -21,8 +21,19 @@ constexpr int kResErr = kResCol + kLadder * kMaxKrylov;
 constexpr int kResFlag = kResErr + kLadder;   // .x != 0: a G cell pass gave up waiting for a block copy
 constexpr int kResSize = kResFlag + 1;
 
+// The Krylov basis as integers on per-group exponents (see gs_dots_kernel).
+struct KrylovBasis {
+    int4* V;          // [m+1][tiles][rows per thread][threads]
+    int* e;           // [m+1][tiles][threads]
+    int64_t stride;   // elements of a vector
+    int64_t estride;  // exponents of a vector
+    int64_t tiles;
+};
+
 struct ArnoldiWork {
-    double2* V;          // [m+1][N][n] Krylov basis
+    KrylovBasis B;       // the Krylov basis
+    int rows;            // rows of a basis tile per thread
+    double2* vd;         // [N][n] FP64 form: the vector G is applied to, and the raw vector G v
     double2* z;          // [N][n] cell-pass output
     double2* cpartial;   // reduction partials
     double2* S;          // [n][n] projector overlaps
@@ -34,6 +45,7 @@ struct ArnoldiWork {
     double2* err;        // [kLadder] error estimates over beta (in res)
     double2* c1;         // inner products and norm of the first Gram-Schmidt pass
     double2* c2;         // the same for the second pass
+    double* f;           // scales of the stored vectors, then beta
     float2* v32;         // [N][n] complex64 copy of the vector G is applied to (mixed form)
     float2* z32;         // [N][n] complex64 cell-pass output (mixed form)
     float2* phi32;       // [N][n] complex64 copy of the frozen orbitals (mixed-form projector)
@@ -47,7 +59,6 @@ struct ArnoldiWork {
     const float4* gb;    // frozen per-cell blocks of the G cell pass for this call, else null
     float4* vh32;        // [nh][n/2] C v at the hanging points (pipelined G cell pass)
     double* bulk_err;    // res[kResFlag].x
-    int64_t stride;      // N * n
 };
 
 int cdot(const double2* A, int na, const double2* B, int nb, const double* w, int64_t rows, int diag,

@@ -70,6 +70,14 @@ __device__ __forceinline__ void fx_mad(FxAcc& a, Fx u, Fx v) {
     asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a.x) : "r"(u.h), "r"(v.l));
     asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a.x) : "r"(u.l), "r"(v.h));
 }
+// The same with a factor u in constant memory, which the instruction takes as
+// its operand (written as above it is moved to a register first: 17 % more
+// instructions in the cell pass; the vector passes have 15 % fewer as above).
+__device__ __forceinline__ void fx_mad_const(FxAcc& a, Fx u, Fx v) {
+    a.hh += static_cast<long long>(u.h) * v.h;
+    a.x += static_cast<long long>(u.h) * v.l;
+    a.x += static_cast<long long>(u.l) * v.h;
+}
 
 // Moves the high word of x to hh.  x holds 16 h l terms of at most 2^59 (8
 // products) between two calls.

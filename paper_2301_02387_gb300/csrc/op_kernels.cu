@@ -240,6 +240,9 @@ __global__ void __launch_bounds__(256) g_cell_kernel(CellArgs a, const double2* 
     }
 }
 
+int launch_cell_fx(const afem_mesh* m, const CellArgs& a, const double* x, const double2* U, double* y, int ncol,
+                   cudaStream_t s);
+
 // velocity != 0: E holds the vector potential A of the velocity gauge (the
 // field term is then -i A . grad instead of E . r).
 int launch_g_cell(const afem_mesh* m, const double* E, const double2* v, const double2* U, double2* z, int n,
@@ -262,11 +265,12 @@ int launch_g_cell(const afem_mesh* m, const double* E, const double2* v, const d
     const unsigned grid = unsigned(m->dev.ncell);
     AFEM_CUDA_TRY(cudaMemsetAsync(z, 0, size_t(m->dev.n_master) * n * sizeof(double2), s));
     if (grid == 0) return AFEM_OK;
+    if (!a.vg && !m->ecs_on)   // length gauge, unscaled: contractions on the integer pipe
+        return launch_cell_fx(m, a, reinterpret_cast<const double*>(v), U, reinterpret_cast<double*>(z), 2 * n, s);
     switch (p) {
 #define AFEM_CASE(PP)                                                                          \
     case PP: {                                                                                 \
-        auto k = a.vg ? g_cell_kernel<PP, true> : g_cell_kernel<PP, false>;                    \
-        if (m->ecs_on) k = g_cell_kernel<PP, false, true>;                                     \
+        auto k = m->ecs_on ? g_cell_kernel<PP, false, true> : g_cell_kernel<PP, true>;         \
         if (smem > 48 * 1024)                                                                  \
             AFEM_CUDA_TRY(allow_dyn_smem(k));                                    \
         AFEM_LAUNCH((k), grid, 256, smem, s, a, v, U, z, n);                                              \
@@ -377,7 +381,7 @@ int launch_stiffness(const afem_mesh* m, const double* x, double* y, int nv, int
     a.with_pot = 0;
     a.masked = masked;
     AFEM_CUDA_TRY(cudaMemsetAsync(y, 0, size_t(m->dev.n_master) * nv * sizeof(double), s));
-    return launch_cell_op<double>(m, a, x, y, nv, s);
+    return launch_cell_fx(m, a, x, nullptr, y, nv, s);
 }
 
 int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int masked, cudaStream_t s,
@@ -396,7 +400,9 @@ int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void
         for (int i = 0; i < 3; ++i) a.E[i] = E ? E[i] : 0.0;
         auto* yy = static_cast<double2*>(y);
         AFEM_CUDA_TRY(cudaMemsetAsync(yy, 0, size_t(N) * nv * sizeof(double2), s));
-        int rc = launch_cell_op<double2>(m, a, static_cast<const double2*>(x), yy, nv, s);
+        int rc = m->ecs_on ? launch_cell_op<double2>(m, a, static_cast<const double2*>(x), yy, nv, s)
+                           : launch_cell_fx(m, a, static_cast<const double*>(x), nullptr, static_cast<double*>(y),
+                                            2 * nv, s);
         if (rc) return rc;
         return launch_scale_rows<double2>(yy, m->dev.ml_inv, N, nv, s);
     }
@@ -420,7 +426,7 @@ int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void
         a.masked = 0;
         auto* yy = static_cast<double*>(y);
         AFEM_CUDA_TRY(cudaMemsetAsync(yy, 0, size_t(N) * nv * sizeof(double), s));
-        return launch_cell_op<double>(m, a, static_cast<const double*>(x), yy, nv, s);
+        return launch_cell_fx(m, a, static_cast<const double*>(x), nullptr, yy, nv, s);
     }
     if (kind == AFEM_OP_POS || kind == AFEM_OP_FORCE) {   // y = M_L^-1 F[e.r] x or M_L^-1 F[e.force] x, masked
         a.c_kin = 0.0;

@@ -191,7 +191,9 @@ int upload_mesh(afem_mesh* m);
 void free_device_mesh(DeviceMesh& d);
 int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void* y, int nvec,
                     cudaStream_t s);
-int launch_stiffness(const afem_mesh* m, const double* x, double* y, int nv, int masked, cudaStream_t s);
+// y = A x (y_zero: y is already cleared)
+int launch_stiffness(const afem_mesh* m, const double* x, double* y, int nv, int masked, cudaStream_t s,
+                     bool y_zero = false);
 int poisson_batch(afem_mesh* m, const double2* phi, int n, double* W, double rtol, int max_it, int warm,
                   int* iters_out, double* relres_out, cudaStream_t s);
 int poisson_batch_mixed(afem_mesh* m, const double2* phi, int n, double* W, double rtol, int max_it, int warm,

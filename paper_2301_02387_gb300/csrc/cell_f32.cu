@@ -42,6 +42,7 @@ struct CellArgs32 {
     float E[3];
     float Avec[3];              // vector potential (vg != 0)
     int masked;
+    int y_zero;                 // (host) the output is already cleared
     int vg;                     // velocity gauge: -i A . grad in the G pass (generic kernel only)
     // G pass: the mean fields at the hanging points, [nh][n^2] complex64 rows
     // (C U, formed once per propagation); null: interpolated from the masters
@@ -1011,7 +1012,7 @@ static int launch32(const afem_mesh* m, const CellArgs32& a, const T* x, const f
     const int nn = (p + 1) * (p + 1) * (p + 1);
     const size_t smem = size_t(nn) * nv * sizeof(T) + ((G && U) ? size_t(nn) * nv * nv * sizeof(float2) : 0);
     const unsigned grid = unsigned(m->dev.ncell);
-    AFEM_CUDA_TRY(cudaMemsetAsync(y, 0, size_t(m->dev.n_master) * nv * sizeof(T), s));
+    if (!a.y_zero) AFEM_CUDA_TRY(cudaMemsetAsync(y, 0, size_t(m->dev.n_master) * nv * sizeof(T), s));
     if (grid == 0) return AFEM_OK;
     switch (p) {
 #define AFEM_CASE(PP)                                                                          \
@@ -1220,7 +1221,7 @@ static int launch32v(const afem_mesh* m, const CellArgs32& a, const float* x, co
     const int nn = (p + 1) * (p + 1) * (p + 1);
     const int L4 = L / 4;
     const unsigned grid = unsigned(m->dev.ncell);
-    AFEM_CUDA_TRY(cudaMemsetAsync(y, 0, size_t(m->dev.n_master) * L * sizeof(float), s));
+    if (!a.y_zero) AFEM_CUDA_TRY(cudaMemsetAsync(y, 0, size_t(m->dev.n_master) * L * sizeof(float), s));
     if (grid == 0) return AFEM_OK;
     const float4* x4 = reinterpret_cast<const float4*>(x);
     float4* y4 = reinterpret_cast<float4*>(y);
@@ -1288,9 +1289,10 @@ static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // (x = p, masked), for nv in {4, 8, 16} on the four-lane path; returns
 // AFEM_EINVAL when they are asked for outside it.
 int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int masked, cudaStream_t s,
-                       double* pap_slots) {
+                       double* pap_slots, bool y_zero) {
     CellArgs32 a = make_cell_args32(m);
     a.masked = masked;
+    a.y_zero = y_zero ? 1 : 0;
     const bool quads = nv % 4 == 0 && aligned16(x) && aligned16(y);
     if (pap_slots) {
         if (!quads || !(nv == 4 || nv == 8 || nv == 16) || m->cell32_variant == 1)

@@ -375,17 +375,17 @@ static int launch_scale_rows(T* y, const double* s, int64_t n, int nv, cudaStrea
     return AFEM_OK;
 }
 
-int launch_stiffness(const afem_mesh* m, const double* x, double* y, int nv, int masked, cudaStream_t s) {
+int launch_stiffness(const afem_mesh* m, const double* x, double* y, int nv, int masked, cudaStream_t s, bool y_zero) {
     CellArgs a = make_cell_args(m);
     a.c_kin = 1.0;
     a.with_pot = 0;
     a.masked = masked;
-    AFEM_CUDA_TRY(cudaMemsetAsync(y, 0, size_t(m->dev.n_master) * nv * sizeof(double), s));
+    if (!y_zero) AFEM_CUDA_TRY(cudaMemsetAsync(y, 0, size_t(m->dev.n_master) * nv * sizeof(double), s));
     return launch_cell_fx(m, a, x, nullptr, y, nv, s);
 }
 
 int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int masked, cudaStream_t s,
-                       double* pap_slots = nullptr);
+                       double* pap_slots = nullptr, bool y_zero = false);
 int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const float2* U, float2* z, int n,
                     cudaStream_t s, int velocity = 0, const float2* U_hang = nullptr);
 

@@ -79,8 +79,8 @@ __device__ __forceinline__ void fx_mad_const(FxAcc& a, Fx u, Fx v) {
     a.x += static_cast<long long>(u.l) * v.h;
 }
 
-// Moves the high word of x to hh.  x holds 16 h l terms of at most 2^59 (8
-// products) between two calls.
+// Moves the high word of x to hh.  A product adds less than 2^60 - 2^27 to x, so
+// x holds 8 products from zero, or 7 and what a carry left (below 2^32).
 __device__ __forceinline__ void fx_carry(FxAcc& a) {
     a.hh += a.x >> 32;
     a.x &= 0xFFFFFFFFll;

@@ -18,6 +18,7 @@
 
 #include "afem_internal.h"
 #include "cell_common.cuh"
+#include "fixed64.cuh"
 #include "vec_common.cuh"
 
 namespace afem {
@@ -27,8 +28,12 @@ constexpr int kNlm = kMultipoleTerms;
 constexpr int kMomTile = 32;
 static int mom_blocks() { return 2 * device_sms(); }   // moment partial rows: 2 blocks per SM
 int mom_blocks_count() { return mom_blocks(); }
-__constant__ double c_sh_norm[kNlm];       // factor applied to C_lm / S_lm at index l*l + l + |m|
+__constant__ double c_sh_norm2[kNlm];      // squared normalisation of C_lm / S_lm at index l*l + l + m
 __constant__ double c_sh_irreg[kLmax + 1];  // 4 pi / (2l + 1)
+// recurrence in l at order m: C_lm = a z C_{l-1,m} - b r^2 C_{l-2,m} with
+// a = (2l-1)/(l-m), b = (l+m-1)/(l-m) (float64 divisions in the kernels took
+// most of the harmonics' time)
+__constant__ double c_sh_a[(kLmax + 1) * (kLmax + 1)], c_sh_b[(kLmax + 1) * (kLmax + 1)];   // [l][m]
 
 // Uploads the solid-harmonic normalisations once per device (synchronous
 // copies; serialised across host threads).
@@ -40,95 +45,67 @@ int ensure_sh_tables() {
     std::lock_guard<std::mutex> lock(mu);
     if (dev < 64 && done[dev]) return AFEM_OK;
     double norm[kNlm], irr[kLmax + 1];
+    double ca[(kLmax + 1) * (kLmax + 1)] = {}, cb[(kLmax + 1) * (kLmax + 1)] = {};
+    for (int l = 0; l <= kLmax; ++l)
+        for (int m = 0; m < l; ++m) {
+            ca[l * (kLmax + 1) + m] = double(2 * l - 1) / (l - m);
+            cb[l * (kLmax + 1) + m] = double(l + m - 1) / (l - m);
+        }
     for (int l = 0; l <= kLmax; ++l) {
         irr[l] = 4.0 * M_PI / (2 * l + 1);
         for (int m = -l; m <= l; ++m) {
             const int am = m < 0 ? -m : m;
             double ratio = 1.0;   // (l-|m|)! / (l+|m|)!
             for (int t = l - am + 1; t <= l + am; ++t) ratio /= t;
-            double N = std::sqrt((2 * l + 1) / (4.0 * M_PI) * ratio);
-            norm[l * l + l + m] = am == 0 ? N : std::sqrt(2.0) * N;
+            norm[l * l + l + m] = (2 * l + 1) / (4.0 * M_PI) * ratio * (am == 0 ? 1.0 : 2.0);
         }
     }
-    AFEM_CUDA_TRY(cudaMemcpyToSymbol(c_sh_norm, norm, sizeof(norm)));
+    AFEM_CUDA_TRY(cudaMemcpyToSymbol(c_sh_norm2, norm, sizeof(norm)));
     AFEM_CUDA_TRY(cudaMemcpyToSymbol(c_sh_irreg, irr, sizeof(irr)));
+    AFEM_CUDA_TRY(cudaMemcpyToSymbol(c_sh_a, ca, sizeof(ca)));
+    AFEM_CUDA_TRY(cudaMemcpyToSymbol(c_sh_b, cb, sizeof(cb)));
     if (dev < 64) done[dev] = true;
     return AFEM_OK;
 }
 
-// Real regular solid harmonics R[l*l + l + m] = r^l Y_lm(x^), l <= kLmax.
-// With C_lm + i S_lm = r^l P_l^m(cos t) e^{i m p}:
+// Real regular solid harmonics without their normalisation, R[l*l + l + m] = C_lm
+// and R[l*l + l - m] = S_lm, l <= kLmax (r^l Y_lm = N C_l0, sqrt2 N C_lm, sqrt2 N
+// S_lm; the squared factors enter the moments).  With C_lm + i S_lm = r^l
+// P_l^m(cos t) e^{i m p}:
 //   C_mm + i S_mm = -(2m-1) (x + i y) (C_{m-1,m-1} + i S_{m-1,m-1}),
-//   C_{m+1,m} = (2m+1) z C_mm,
-//   C_lm = ((2l-1) z C_{l-1,m} - (l+m-1) r^2 C_{l-2,m}) / (l - m),
-// and Y_l0 = N_l0 C_l0, Y_lm = sqrt2 N_lm C_lm, Y_l,-m = sqrt2 N_lm S_lm.
+//   C_lm = ((2l-1) z C_{l-1,m} - (l+m-1) r^2 C_{l-2,m}) / (l - m).
+// One order m, from C_mm, S_mm.
+__device__ __forceinline__ void solid_harmonics_l(double z, double r2, int m, double cmm, double smm, double* R) {
+    double c2 = 0.0, s2 = 0.0, c1 = cmm, s1 = smm;
+    {
+        const int i = m * m + m;
+        R[i + m] = cmm;
+        if (m > 0) R[i - m] = smm;
+    }
+    for (int l = m + 1; l <= kLmax; ++l) {
+        const double az = c_sh_a[l * (kLmax + 1) + m] * z, br = c_sh_b[l * (kLmax + 1) + m] * r2;
+        const double c = fma(az, c1, -br * c2), t = fma(az, s1, -br * s2);
+        const int i = l * l + l;
+        R[i + m] = c;
+        if (m > 0) R[i - m] = t;
+        c2 = c1;
+        s2 = s1;
+        c1 = c;
+        s1 = t;
+    }
+}
+__device__ __forceinline__ void solid_harmonics_mm(double x, double y, int m, double& cmm, double& smm) {
+    const double f = -(2 * m + 1);   // from order m to m + 1
+    const double nc = f * (x * cmm - y * smm);
+    smm = f * (x * smm + y * cmm);
+    cmm = nc;
+}
 __device__ void regular_solid_harmonics(double x, double y, double z, double* R) {
     const double r2 = x * x + y * y + z * z;
     double cmm = 1.0, smm = 0.0;
     for (int m = 0; m <= kLmax; ++m) {
-        double c2 = 0.0, s2 = 0.0, c1 = cmm, s1 = smm;
-        {
-            const int i = m * m + m;
-            R[i + m] = c_sh_norm[i + m] * cmm;
-            if (m > 0) R[i - m] = c_sh_norm[i + m] * smm;
-        }
-        for (int l = m + 1; l <= kLmax; ++l) {
-            double c, s;
-            if (l == m + 1) {
-                c = (2 * m + 1) * z * c1;
-                s = (2 * m + 1) * z * s1;
-            } else {
-                c = ((2 * l - 1) * z * c1 - (l + m - 1) * r2 * c2) / (l - m);
-                s = ((2 * l - 1) * z * s1 - (l + m - 1) * r2 * s2) / (l - m);
-            }
-            const int i = l * l + l;
-            R[i + m] = c_sh_norm[i + m] * c;
-            if (m > 0) R[i - m] = c_sh_norm[i + m] * s;
-            c2 = c1;
-            s2 = s1;
-            c1 = c;
-            s1 = s;
-        }
-        const double nc = -(2 * m + 1) * (x * cmm - y * smm);
-        const double ns = -(2 * m + 1) * (x * smm + y * cmm);
-        cmm = nc;
-        smm = ns;
-    }
-}
-
-// One order m of the same harmonics (l = m..kLmax): C_mm, S_mm by the same
-// recurrence in m, then the recurrence in l; lets several threads share a point.
-__device__ void solid_harmonics_order(double x, double y, double z, int m, double* R) {
-    const double r2 = x * x + y * y + z * z;
-    double cmm = 1.0, smm = 0.0;
-    for (int q = 0; q < m; ++q) {
-        const double nc = -(2 * q + 1) * (x * cmm - y * smm);
-        const double ns = -(2 * q + 1) * (x * smm + y * cmm);
-        cmm = nc;
-        smm = ns;
-    }
-    double c2 = 0.0, s2 = 0.0, c1 = cmm, s1 = smm;
-    {
-        const int i = m * m + m;
-        R[i + m] = c_sh_norm[i + m] * cmm;
-        if (m > 0) R[i - m] = c_sh_norm[i + m] * smm;
-    }
-    for (int l = m + 1; l <= kLmax; ++l) {
-        double c, s;
-        if (l == m + 1) {
-            c = (2 * m + 1) * z * c1;
-            s = (2 * m + 1) * z * s1;
-        } else {
-            c = ((2 * l - 1) * z * c1 - (l + m - 1) * r2 * c2) / (l - m);
-            s = ((2 * l - 1) * z * s1 - (l + m - 1) * r2 * s2) / (l - m);
-        }
-        const int i = l * l + l;
-        R[i + m] = c_sh_norm[i + m] * c;
-        if (m > 0) R[i - m] = c_sh_norm[i + m] * s;
-        c2 = c1;
-        s2 = s1;
-        c1 = c;
-        s1 = s;
+        solid_harmonics_l(z, r2, m, cmm, smm, R);
+        solid_harmonics_mm(x, y, m, cmm, smm);
     }
 }
 
@@ -147,24 +124,44 @@ struct PointArgs {
     double cx, cy, cz;      // expansion centre
 };
 
-// RHS b = 4 pi C^T (m_f o rho) (atomics into zeroed b) and per-block moment partials.
+// RHS b = 4 pi C^T (m_f o rho) (atomics into zeroed b) and per-block partials of
+// the (unnormalised) moments sum_f m_f rho_f R_lm(x_f).
 // Per tile of kMomTile support points, every phase is spread over the block:
 // (point, orbital) items stage the orbital values (hanging points through C),
-// (point, column) items form m_f rho_c and the right-hand side, then the
-// harmonics and the moment contraction.
-__global__ void __launch_bounds__(256) pair_rhs_moments_kernel(PointArgs a, double* __restrict__ b,
-                                                               double* __restrict__ qpart) {
+// (point, column) items form m_f rho_c and the right-hand side; seven threads
+// per point form the harmonics, orders m and 12 - m each (14 steps for all).
+// The contraction over the tile's points, 169 n^2 products per point, runs on
+// the integer pipe (fixed64.cuh; groups: the 32 points of one harmonic, and of
+// one column), each thread 4 harmonics x 4 columns in registers.  As FP64
+// multiply-adds with both factors from shared memory, and divisions in the
+// harmonics, the 830,209 points x 16 columns of the H2 benchmark took 13.9 ms;
+// now 7.1 ms.
+constexpr int kMomLm4 = (kNlm + 3) / 4 * 4;   // harmonics padded to quads
+constexpr int kMomRow = kMomLm4 + 2;          // row of a point (8-byte words; even, off the bank period)
+static size_t mom_smem(int ncol) {
+    const int nc4 = (ncol + 3) / 4 * 4;
+    return (size_t(kMomTile) * kMomRow + size_t(kMomTile) * nc4 + size_t(kMomLm4) * nc4) * sizeof(double) +
+           (size_t(kMomLm4) + nc4) * sizeof(int);
+}
+__global__ void __launch_bounds__(256, 2) pair_rhs_moments_kernel(PointArgs a, double* __restrict__ b,
+                                                                  double* __restrict__ qpart) {
     extern __shared__ __align__(16) double smem_d[];
-    double* s_R = smem_d;                          // [kMomTile][kNlm]
-    double* s_w = s_R + kMomTile * kNlm;           // [kMomTile][ncol]
-    double* s_Q = s_w + kMomTile * a.ncol;         // [kNlm][ncol]
-    __shared__ double4 s_pt[kMomTile];             // point relative to the centre, valid flag
+    const int ncol = a.ncol, n = a.n, nc4 = (ncol + 3) / 4 * 4;
+    double* s_R = smem_d;                          // [kMomTile][kMomRow] harmonics, then their integers
+    double* s_w = s_R + kMomTile * kMomRow;        // [kMomTile][nc4] m_f rho_c, then their integers
+    double* s_Q = s_w + kMomTile * nc4;            // [kMomLm4][nc4] the block's moments
+    int* s_eR = reinterpret_cast<int*>(s_Q + kMomLm4 * nc4);   // [kMomLm4] group exponents
+    int* s_ew = s_eR + kMomLm4;                    // [nc4]
+    int2* i_R = reinterpret_cast<int2*>(s_R);      // (l, h)
+    int2* i_w = reinterpret_cast<int2*>(s_w);
+    __shared__ double4 s_pt[kMomTile];             // point relative to the centre
     __shared__ double2 s_ph[kMomTile][8];          // orbital values at the tile's points
     __shared__ double s_mf[kMomTile];
     __shared__ int s_col[64];                      // column c -> r | s << 8 | part << 16
-    const int ncol = a.ncol, n = a.n;
     const int tid = threadIdx.x;
-    for (int o = tid; o < kNlm * ncol; o += blockDim.x) s_Q[o] = 0.0;
+    for (int o = tid; o < kMomLm4 * nc4; o += blockDim.x) s_Q[o] = 0.0;
+    for (int o = tid; o < kMomTile * (kMomRow - kNlm); o += blockDim.x)   // the padding stays zero
+        s_R[(o / (kMomRow - kNlm)) * kMomRow + kNlm + o % (kMomRow - kNlm)] = 0.0;
     if (tid == 0) {
         int c = 0;
         for (int r = 0; r < n; ++r) s_col[c++] = r | (r << 8);
@@ -197,27 +194,17 @@ __global__ void __launch_bounds__(256) pair_rhs_moments_kernel(PointArgs a, doub
         }
         for (int tp = tid; tp < kMomTile; tp += blockDim.x) {
             const int64_t f = tile * kMomTile + tp;
-            if (f < a.N) {
-                s_mf[tp] = a.mf_m[f];
-                s_pt[tp] = make_double4(a.xyz_m[3 * f] - a.cx, a.xyz_m[3 * f + 1] - a.cy, a.xyz_m[3 * f + 2] - a.cz,
-                                        1.0);
-            } else if (f < npts) {
-                const int64_t h = f - a.N;
-                s_mf[tp] = a.mf_h[h];
-                s_pt[tp] = make_double4(a.xyz_h[3 * h] - a.cx, a.xyz_h[3 * h + 1] - a.cy, a.xyz_h[3 * h + 2] - a.cz,
-                                        1.0);
-            } else {
-                s_mf[tp] = 0.0;
-                s_pt[tp] = make_double4(0.0, 0.0, 0.0, 0.0);
-            }
+            const double* x = f < a.N ? a.xyz_m + 3 * f : f < npts ? a.xyz_h + 3 * (f - a.N) : nullptr;
+            s_mf[tp] = !x ? 0.0 : f < a.N ? a.mf_m[f] : a.mf_h[f - a.N];
+            s_pt[tp] = x ? make_double4(x[0] - a.cx, x[1] - a.cy, x[2] - a.cz, 0.0) : make_double4(0.0, 0.0, 0.0, 0.0);
         }
         __syncthreads();
         // m_f rho_c and the right-hand side through C^T
-        for (int it = tid; it < kMomTile * ncol; it += blockDim.x) {
-            const int tp = it / ncol, c = it - tp * ncol;
+        for (int it = tid; it < kMomTile * nc4; it += blockDim.x) {
+            const int tp = it / nc4, c = it - tp * nc4;
             const int64_t f = tile * kMomTile + tp;
             double wv = 0.0;
-            if (f < npts) {
+            if (f < npts && c < ncol) {
                 const int code = s_col[c];
                 const double2 x = s_ph[tp][code & 0xFF], y = s_ph[tp][(code >> 8) & 0xFF];
                 const double rho = (code >> 16) ? x.x * y.y - x.y * y.x : x.x * y.x + x.y * y.y;
@@ -233,47 +220,96 @@ __global__ void __launch_bounds__(256) pair_rhs_moments_kernel(PointArgs a, doub
                         atomicAdd(&b[int64_t(a.hm[e]) * ncol + c], fpi * a.hw[e] * wv);
                 }
             }
-            s_w[tp * ncol + c] = wv;
+            s_w[it] = wv;
         }
-        __syncthreads();
-        // harmonics of the tile: 8 threads per point, orders m and m + 8
-        for (int it = tid; it < kMomTile * 8; it += blockDim.x) {
-            const int tp = it >> 3, j = it & 7;
+        // harmonics of the tile (points beyond the last carry m_f rho = 0)
+        if (tid < kMomTile * 7) {
+            const int tp = tid / 7, j = tid - tp * 7;
             const double4 q = s_pt[tp];
-            double* Rr = s_R + tp * kNlm;
-            for (int m = j; m <= kLmax; m += 8) {
-                if (q.w != 0.0) {
-                    solid_harmonics_order(q.x, q.y, q.z, m, Rr);
-                } else {
-                    for (int l = m; l <= kLmax; ++l) {
-                        Rr[l * l + l + m] = 0.0;
-                        if (m > 0) Rr[l * l + l - m] = 0.0;
-                    }
-                }
+            const double r2 = q.x * q.x + q.y * q.y + q.z * q.z;
+            double cmm = 1.0, smm = 0.0;
+            for (int m = 0; m <= kLmax - j; ++m) {
+                if (m == j || m == kLmax - j) solid_harmonics_l(q.z, r2, m, cmm, smm, s_R + tp * kMomRow);
+                solid_harmonics_mm(q.x, q.y, m, cmm, smm);
             }
         }
         __syncthreads();
-        for (int o = tid; o < kNlm * ncol; o += blockDim.x) {
-            const int lm = o / ncol, c = o - lm * ncol;
-            double acc = s_Q[o];
-            for (int t = 0; t < kMomTile; ++t) acc = fma(s_R[t * kNlm + lm], s_w[t * ncol + c], acc);
-            s_Q[o] = acc;
+        // integers in place, one harmonic or column per thread (32 points each)
+        for (int o = tid; o < kMomLm4 + nc4; o += blockDim.x) {
+            const bool isR = o < kMomLm4;
+            const int ld = isR ? kMomRow : nc4, c = isR ? o : o - kMomLm4;
+            double* v = (isR ? s_R : s_w) + c;
+            unsigned e = 0u;
+            for (int t = 0; t < kMomTile; ++t) e = max(e, fx_expbits(v[t * ld]));
+            const int eg = max(int(e >> 20), kFxMinExp);
+            for (int t = 0; t < kMomTile; ++t) {
+                const Fx f = fx_make(v[t * ld], eg);
+                reinterpret_cast<int2*>(v)[t * ld] = make_int2(f.l, f.h);
+            }
+            (isR ? s_eR : s_ew)[c] = e == kFxExpMask ? 0x7FFF : eg;
+        }
+        __syncthreads();
+        for (int it = tid; it < kMomLm4 / 4 * (nc4 / 4); it += blockDim.x) {
+            const int g = it / (nc4 / 4), lm = 4 * g, c = 4 * (it - g * (nc4 / 4));
+            FxAcc acc[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = FxAcc{0, 0};
+            for (int t0 = 0; t0 < kMomTile; t0 += 4) {   // 4 products between carries
+#pragma unroll 2
+                for (int t = t0; t < t0 + 4; ++t) {
+                    const int4* pr = reinterpret_cast<const int4*>(i_R + t * kMomRow + lm);
+                    const int4* pw = reinterpret_cast<const int4*>(i_w + t * nc4 + c);
+                    const int4 r0 = pr[0], r1 = pr[1], w0 = pw[0], w1 = pw[1];
+                    const Fx fr[4] = {{r0.y, r0.x}, {r0.w, r0.z}, {r1.y, r1.x}, {r1.w, r1.z}};
+                    const Fx fw[4] = {{w0.y, w0.x}, {w0.w, w0.z}, {w1.y, w1.x}, {w1.w, w1.z}};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) fx_mad(acc[i][j], fr[i], fw[j]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) fx_carry(acc[i][j]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    double& q = s_Q[(lm + i) * nc4 + c + j];
+                    q = fma(fx_value(acc[i][j]), fx_scale(s_eR[lm + i] + s_ew[c + j]), q);
+                }
         }
     }
     __syncthreads();
-    for (int o = tid; o < kNlm * ncol; o += blockDim.x) qpart[int64_t(blockIdx.x) * kNlm * ncol + o] = s_Q[o];
+    for (int o = tid; o < kNlm * ncol; o += blockDim.x)
+        qpart[int64_t(blockIdx.x) * kNlm * ncol + o] = s_Q[(o / ncol) * nc4 + o % ncol];
 }
 
-__global__ void finalize_columns_kernel(const double* __restrict__ partial, int nblk, int k,
-                                        double* __restrict__ out) {
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        double acc = 0.0;
-        for (int b = 0; b < nblk; ++b) acc += partial[int64_t(b) * k + c];
-        out[c] = acc;
+// q[lm][c] = squared normalisation x the sum of the blocks' partials: 32 values
+// per block of 256 threads, 8 threads each (one block over all values took
+// 410 us for 2,704 values of 304 rows).
+__global__ void __launch_bounds__(256) moments_finalize_kernel(const double* __restrict__ partial, int nblk, int ncol,
+                                                               double* __restrict__ q) {
+    __shared__ double s[256];
+    const int k = kNlm * ncol, o = blockIdx.x * 32 + (threadIdx.x & 31), r = threadIdx.x >> 5;
+    double acc = 0.0;
+    if (o < k) {
+#pragma unroll 8
+        for (int b = r; b < nblk; b += 8) acc += partial[int64_t(b) * k + o];
+    }
+    s[threadIdx.x] = acc;
+    __syncthreads();
+    if (r == 0 && o < k) {
+        for (int i = 1; i < 8; ++i) acc += s[threadIdx.x + 32 * i];
+        q[o] = acc * c_sh_norm2[o / ncol];
     }
 }
 
-// Dirichlet data g at the surface masters from the moments; written into x.
+// Dirichlet data g at the surface masters from the moments (with the squared
+// normalisations of the harmonics); written into x.
 __global__ void multipole_bc_kernel(const double* __restrict__ q, int ncol, const double* __restrict__ xyz,
                                     int64_t n_int, int64_t N, double cx, double cy, double cz,
                                     double* __restrict__ x) {
@@ -721,12 +757,12 @@ int poisson_rhs_bc(afem_mesh* m, const double2* phi, int n, double* W, double* b
     const double c0 = 0.5 * (m->desc.lo + m->desc.hi);
     a.cx = a.cy = a.cz = c0;
     AFEM_CUDA_TRY(cudaMemsetAsync(b, 0, size_t(D.n_master) * ncol * sizeof(double), s));
-    const size_t smem = (size_t(kMomTile) * kNlm + size_t(kMomTile) * ncol + size_t(kNlm) * ncol) * sizeof(double);
+    const size_t smem = mom_smem(ncol);
     AFEM_CUDA_TRY(allow_dyn_smem(pair_rhs_moments_kernel));
     const int nblk = mom_blocks();
     AFEM_LAUNCH((pair_rhs_moments_kernel), nblk, 256, smem, s, a, b, qpart);
     AFEM_CUDA_TRY(cudaGetLastError());
-    AFEM_LAUNCH((finalize_columns_kernel), 1, 256, 0, s, qpart, nblk, kNlm * ncol, q);
+    AFEM_LAUNCH((moments_finalize_kernel), (kNlm * ncol + 31) / 32, 256, 0, s, qpart, nblk, ncol, q);
     AFEM_CUDA_TRY(cudaGetLastError());
     const int64_t nb = D.n_master - D.n_interior;
     if (nb > 0) {
@@ -859,10 +895,10 @@ int multipole_boundary(afem_mesh* m, const double2* phi, int n, double* W, doubl
     a.hw = D.hang_w;
     const double c0 = 0.5 * (m->desc.lo + m->desc.hi);
     a.cx = a.cy = a.cz = c0;
-    const size_t smem = (size_t(kMomTile) * kNlm + size_t(kMomTile) * ncol + size_t(kNlm) * ncol) * sizeof(double);
+    const size_t smem = mom_smem(ncol);
     AFEM_CUDA_TRY(allow_dyn_smem(pair_rhs_moments_kernel));
     AFEM_LAUNCH((pair_rhs_moments_kernel), nblk, 256, smem, s, a, static_cast<double*>(nullptr), qpart);
-    AFEM_LAUNCH((finalize_columns_kernel), 1, 256, 0, s, qpart, nblk, kNlm * ncol, q);
+    AFEM_LAUNCH((moments_finalize_kernel), (kNlm * ncol + 31) / 32, 256, 0, s, qpart, nblk, ncol, q);
     AFEM_CUDA_TRY(cudaGetLastError());
     const int64_t nb = D.n_master - D.n_interior;
     if (nb > 0) {

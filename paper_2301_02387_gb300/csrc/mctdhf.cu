@@ -651,9 +651,11 @@ static void finalize_cpartials(const double2* partial, int nblk, int k, double2*
 __global__ void csum_blocks_kernel(const double2* __restrict__ partial, int nblk, int k, double2* __restrict__ out) {
     for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < k; o += gridDim.x * blockDim.x) {
         double x = 0.0, y = 0.0;
-        for (int b = 0; b < nblk; ++b) {
-            x += partial[int64_t(b) * k + o].x;
-            y += partial[int64_t(b) * k + o].y;
+#pragma unroll 8
+        for (int b = 0; b < nblk; ++b) {   // (loads of eight rows in flight)
+            const double2 v = partial[int64_t(b) * k + o];
+            x += v.x;
+            y += v.y;
         }
         out[o] = make_double2(x, y);
     }
@@ -672,7 +674,8 @@ static int pair_integrals(const afem_mesh* m, const double2* phi, const double* 
                           double2* partial, double2* X, double2* eri, int* tc_status, cudaStream_t s) {
     const DeviceMesh& D = m->dev;
     const int nn = n * n;
-    const int iblk = int_blocks();
+    // the tensor-core blocks: two resident per SM, each block's sums written once
+    const int iblk = tensor_cores ? 2 * device_sms() : int_blocks();
     if (tensor_cores) {
         const int rc = integrals_tc(m, phi, W, n, partial, iblk, tc_status, s);
         if (rc) return rc;

@@ -571,17 +571,17 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_dots_kernel(const __grid_co
     __shared__ double s_sum[kRedThreads];
     if (!last_block_sum(a.partial, 2 * nv, a.counter, s_sum)) return;
     const double fw = s_f[nv - 1];
-    if (tid < nv) {
-        const double f = s_f[tid] * fw;
-        a.out[tid] = make_double2(f * s_sum[2 * tid], f * s_sum[2 * tid + 1]);
-    }
-    if (tid == 0) {
+    if (tid < 32) {
         double nn = 0.0;
-        for (int i = 0; i < nv; ++i) {
-            const double f = s_f[i] * fw;
-            nn += f * f * (s_sum[2 * i] * s_sum[2 * i] + s_sum[2 * i + 1] * s_sum[2 * i + 1]);
+        if (tid < nv) {
+            const double f = s_f[tid] * fw;
+            const double2 o = make_double2(f * s_sum[2 * tid], f * s_sum[2 * tid + 1]);
+            a.out[tid] = o;
+            nn = o.x * o.x + o.y * o.y;
         }
-        a.out[nv] = make_double2(nn, 0.0);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, off);
+        if (tid == 0) a.out[nv] = make_double2(nn, 0.0);
     }
     if (MODE == 2 && a.S_slots)
         for (int o = tid; o < kOvSlots * 2 * n * n; o += blockDim.x) a.S_slots[o] = 0.0;
@@ -1135,17 +1135,18 @@ static unsigned wave_grid(int64_t tiles, size_t smem) {
     return unsigned(std::max<int64_t>(1, std::min(tiles, cap)));
 }
 
-// Rows of a tile per thread: as many as leave the chip several tiles per SM
-// (4: two float64 additions per vector serve four rows; 1 on small meshes,
-// where blocks in flight count for more).
+// Rows of a tile per thread: as many as leave each SM a tile.  The two float64
+// additions of a group and vector serve all its rows, so fewer rows cost more
+// than idle warps: with four tiles per SM asked for, one orbital on 78,761 points
+// took one row per thread and 24.5 us per inner-product pass (28.5 us at ten
+// vectors and more), with one tile per SM two rows and 14.4 us.
 static int krylov_rows(int64_t N, int n) {
     const int64_t R = kRedThreads / n;
     for (int E = 4; E > 1; E >>= 1)
-        if ((N + E * R - 1) / (E * R) >= 4 * device_sms()) return E;
+        if ((N + E * R - 1) / (E * R) >= device_sms()) return E;
     return 1;
 }
 
-// STAGES: as many as leave two blocks per SM beside the sums of nv vectors.
 template <int E, int MODE, int STAGES>
 static int launch_gs_dots_s(const GsDotsArgs& a, cudaStream_t s) {
     constexpr size_t kStage = size_t(STAGES) * kRedThreads * (E * sizeof(int4) + sizeof(int));

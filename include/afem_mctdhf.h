@@ -139,10 +139,11 @@ int afem_convert(const void* x, void* y, int64_t n, int direction, void* stream)
 /* Kernel-class timing (library instrumentation with no counterpart in the
  * paper).  While enabled (process-wide), the library brackets each call of a
  * class's kernels with a pair of CUDA events recorded on the stream the
- * kernels are launched on, and adds the call's algorithmic work: FP64 flops
- * for AFEM_PROF_GS (8 per complex multiply-add with a Krylov vector, 4 per
- * squared norm) and AFEM_PROF_CELL64 (3 (p+1) 2 + 6 per node and real
- * column), bytes for the others (each input and output element once).
+ * kernels are launched on, and adds the call's algorithmic work (whatever pipe
+ * the kernels run it on): flops on float64 quantities for AFEM_PROF_GS (8 per
+ * complex multiply-add with a Krylov vector, 4 per squared norm) and
+ * AFEM_PROF_CELL64 (3 (p+1) 2 + 6 per node and real column), bytes for the
+ * others (each input and output element once).
  * afem_profile_read waits for the recorded events of class `cls` and returns
  * (each pointer may be NULL) the summed event time in milliseconds, the
  * number of bracketed calls and the summed work; reset != 0 clears the class
@@ -189,8 +190,10 @@ int afem_mesh_create_ex(const afem_mesh_desc* desc, int flags, afem_mesh** out);
 int afem_mesh_destroy(afem_mesh* mesh);
 
 /* Kernel-shape options of a mesh (library tuning; no counterpart in the paper).
- * AFEM_OPT_CELL32_VARIANT selects the float32 four-lane cell pass: 0 (default)
- * computes each output node in one thread, 1 computes the 1D contractions
+ * AFEM_OPT_CELL32_VARIANT selects the float32 cell pass: 0 (default) sweeps the
+ * lines of a cell with the 1D matrix in constant memory (operators without mean
+ * fields) or computes each output node in one thread (G, and the CG sweeps'
+ * stiffness with p.Ap), 1 computes the 1D contractions
  * line by line with direction-wise accumulation in shared memory, 2 does the
  * same for the stiffness with one thread per (line, column pair) and the 1D
  * matrix in registers (1, 2 or 4 column quads; other passes as for 0).  All

@@ -1137,9 +1137,8 @@ static unsigned wave_grid(int64_t tiles, size_t smem) {
 
 // Rows of a tile per thread: as many as leave each SM a tile.  The two float64
 // additions of a group and vector serve all its rows, so fewer rows cost more
-// than idle warps: with four tiles per SM asked for, one orbital on 78,761 points
-// took one row per thread and 24.5 us per inner-product pass (28.5 us at ten
-// vectors and more), with one tile per SM two rows and 14.4 us.
+// than idle warps: one orbital on 78,761 points with one row per thread (four
+// tiles per SM) took 24.5 us per inner-product pass, with two rows 17.4 us.
 static int krylov_rows(int64_t N, int n) {
     const int64_t R = kRedThreads / n;
     for (int E = 4; E > 1; E >>= 1)

@@ -12,6 +12,11 @@
 //   -> scatter-add through C^T (atomics) ,
 // and the one-body operator of Eq. discretized_eom, H1~ = 1/2 A + F[V + E.r],
 // is this pass followed by the inverse lumped mass.
+//
+// The unscaled length-gauge operators (the stiffness, H1~ and G) run in
+// cell_fx_kernel, their contractions on the integer pipe; the kernels here carry
+// the velocity gauge, the complex scaling and the pointwise-only operators, with
+// FP64 multiply-adds.
 #include <cmath>
 
 #include "afem_internal.h"

@@ -152,10 +152,6 @@ __device__ __forceinline__ bool last_block_sum(const double* partial, int kout, 
     return true;
 }
 
-// Sum partial[b][c] over blocks b into out[c] (one block, fixed order).
-__global__ void finalize_columns_kernel(const double* __restrict__ partial, int nblk, int k,
-                                        double* __restrict__ out);
-
 // Carve 256-byte-aligned sub-buffers out of one allocation.  A Carver built
 // with a null base only measures: run the same sequence of take() calls once
 // to size the allocation, then again on the real base, so the two can never

@@ -37,9 +37,14 @@ __device__ __forceinline__ double2 to_d2(float2 v) { return make_double2(v.x, v.
 // S[a][b] = sum_k w_k conj(A[k][a]) B[k][b] over rows k < n_rows (w_k = 1 when
 // w is null), reduced in the same launch: partial rows of 2*kout doubles (re,
 // im interleaved); the last block writes out[kout].  diag != 0: only a == b
-// (kout = na), else all na*nb pairs (kout = na*nb <= 256).
+// (kout = na), else all na*nb pairs (kout = na*nb <= 128).  On small meshes
+// latency bounds it, so a thread has kDotRows rows in flight, the threads' sums
+// meet in a tree, and row_blocks() leaves few rows to the last block: 3 x 3 pairs
+// on 102,533 rows took 27 us with four blocks per SM and one row at a time, 19 us
+// with two, 18 us with one.
+constexpr int kDotRows = 4;
 template <typename TB>
-__global__ void cdot_fused_kernel(const double2* __restrict__ A, int na, const TB* __restrict__ B, int nb,
+__global__ void __launch_bounds__(kRedThreads) cdot_fused_kernel(const double2* __restrict__ A, int na, const TB* __restrict__ B, int nb,
                                   const double* __restrict__ w, int64_t n_rows, int diag, double* __restrict__ partial,
                                   unsigned* __restrict__ counter, double2* __restrict__ out) {
     __shared__ double sx[kRedThreads], sy[kRedThreads];
@@ -51,28 +56,45 @@ __global__ void cdot_fused_kernel(const double2* __restrict__ A, int na, const T
         const int o = t % kout, r = t / kout;
         const int ia = diag ? o : o / nb;
         const int ib = diag ? o : o - ia * nb;
-        for (int64_t k = int64_t(blockIdx.x) * R + r; k < n_rows; k += int64_t(gridDim.x) * R) {
-            double2 u = A[k * na + ia];
-            const double2 v = to_d2(B[k * nb + ib]);
-            if (w) {
-                const double wk = w[k];
-                u = make_double2(wk * u.x, wk * u.y);
+        const int64_t step = int64_t(gridDim.x) * R;
+        for (int64_t k0 = int64_t(blockIdx.x) * R + r; k0 < n_rows; k0 += kDotRows * step) {
+            double2 u[kDotRows], v[kDotRows];
+#pragma unroll
+            for (int q = 0; q < kDotRows; ++q) {
+                const int64_t k = k0 + q * step;
+                u[q] = v[q] = make_double2(0.0, 0.0);
+                if (k < n_rows) {
+                    u[q] = A[k * na + ia];
+                    v[q] = to_d2(B[k * nb + ib]);
+                    if (w) {
+                        const double wk = w[k];
+                        u[q] = make_double2(wk * u[q].x, wk * u[q].y);
+                    }
+                }
             }
-            ax = fma(u.x, v.x, fma(u.y, v.y, ax));
-            ay = fma(u.x, v.y, fma(-u.y, v.x, ay));
+#pragma unroll
+            for (int q = 0; q < kDotRows; ++q) {
+                if (k0 + q * step >= n_rows) break;
+                ax = fma(u[q].x, v[q].x, fma(u[q].y, v[q].y, ax));
+                ay = fma(u[q].x, v[q].y, fma(-u[q].y, v[q].x, ay));
+            }
         }
     }
     sx[t] = ax;
     sy[t] = ay;
     __syncthreads();
-    for (int o = t; o < kout; o += blockDim.x) {
-        double x = 0.0, y = 0.0;
-        for (int r = 0; r < R; ++r) {
-            x += sx[o + kout * r];
-            y += sy[o + kout * r];
+    for (int left = R; left > 1;) {   // tree over the rows of threads
+        const int half = (left + 1) >> 1;
+        if (t + half * kout < left * kout) {
+            sx[t] += sx[t + half * kout];
+            sy[t] += sy[t + half * kout];
         }
-        partial[int64_t(blockIdx.x) * 2 * kout + 2 * o] = x;
-        partial[int64_t(blockIdx.x) * 2 * kout + 2 * o + 1] = y;
+        __syncthreads();
+        left = half;
+    }
+    if (t < kout) {
+        partial[int64_t(blockIdx.x) * 2 * kout + 2 * t] = sx[t];
+        partial[int64_t(blockIdx.x) * 2 * kout + 2 * t + 1] = sy[t];
     }
     if (!last_block_sum(partial, 2 * kout, counter, sx)) return;
     for (int o = t; o < kout; o += blockDim.x) out[o] = make_double2(sx[2 * o], sx[2 * o + 1]);
@@ -1073,7 +1095,7 @@ __global__ void hang_rows32_kernel(const float2* __restrict__ U, const int32_t* 
 template <typename TB>
 int cdot_t(const double2* A, int na, const TB* B, int nb, const double* w, int64_t rows, int diag,
            double2* partial, double2* out, unsigned* counter, cudaStream_t s) {
-    AFEM_LAUNCH((cdot_fused_kernel<TB>), red_blocks(), kRedThreads, 0, s, A, na, B, nb, w, rows, diag,
+    AFEM_LAUNCH((cdot_fused_kernel<TB>), row_blocks(rows, diag ? na : na * nb), kRedThreads, 0, s, A, na, B, nb, w, rows, diag,
                 reinterpret_cast<double*>(partial), counter, out);
     AFEM_CUDA_TRY(cudaGetLastError());
     return AFEM_OK;

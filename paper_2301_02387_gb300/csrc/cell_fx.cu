@@ -80,7 +80,7 @@ static size_t cell_fx_smem(int nn, int cpb, int nc, bool pointwise) {
 
 // One component of acc + w u: the real (odd = 0) or the imaginary part.  The
 // operands are selected, with the sign as a bit, so that lanes of both kinds
-// share the two multiply-adds (as two expressions a warp ran all four: 7 complex
+// share the two multiply-adds (as two expressions a warp ran all four: 3 complex
 // orbitals at degree 3 on 4,164 cells took 82 us, now 66 us).
 __device__ __forceinline__ double mean_field_part(double2 w, double2 u, int odd, double acc) {
     const double same = odd ? u.y : u.x, other = odd ? u.x : u.y;
@@ -93,7 +93,7 @@ __device__ __forceinline__ double mean_field_part(double2 w, double2 u, int odd,
 // plus the mean fields U (real columns 2p, 2p + 1: orbital p).  x, y: [N][ncol]
 // doubles; blockIdx.y selects kFxColumns of them.
 template <int P, int PT>
-__global__ void __launch_bounds__(256) cell_fx_kernel(const __grid_constant__ CellArgs a,
+__global__ void __launch_bounds__(256, PT == 2 ? 5 : 1) cell_fx_kernel(const __grid_constant__ CellArgs a,
                                                       const __grid_constant__ FxBasis D, const double* __restrict__ x,
                                                       const double2* __restrict__ U, double* __restrict__ y, int ncol,
                                                       int cpb, int64_t ncell) {

@@ -417,13 +417,12 @@ __global__ void pcg_init_finalize_kernel(const double* __restrict__ partial, int
 }
 
 // ---- fused CG kernels: block partials + last-block finalize (alpha or beta)
-// A thread takes kCgRows rows at a time, their loads in flight together, and two
-// blocks per SM share the work (fewer partial rows for the last block).  On
-// 111,661 x 9 doubles, all of them in L2, p.Ap takes 14 us and the update 27 us;
-// row by row with four blocks per SM they took 18 and 33 us.  What is left is
-// FP64 issue (8 us of the update), the block sums and the last block's.
+// A thread takes kCgRows rows at a time, their loads in flight together, on
+// row_blocks() blocks.  On 111,661 x 9 doubles, all of them in L2, p.Ap took 18 us
+// and the update 33 us row by row with four blocks per SM, 14 and 27 us with two
+// and four rows in flight; one block per SM takes another 3 % off a solve.  What
+// is left is FP64 issue (8 us of the update), the block sums and the last block's.
 constexpr int kCgRows = 4;
-static int cg_blocks() { return std::min(red_blocks(), 2 * device_sms()); }
 // p.Ap per column; the last block sets alpha = rz / pAp for active columns.
 template <typename T>
 __global__ void dot_alpha_kernel(const T* __restrict__ p, const T* __restrict__ Ap, int64_t n, int k,
@@ -876,9 +875,9 @@ int poisson_batch(afem_mesh* m, const double2* phi, int n, double* W, double rto
             ProfScope ps(AFEM_PROF_CELL64, s, double(D.ncell) * p1 * p1 * p1 * k * (3.0 * p1 * 2.0 + 6.0));
             if ((rc = launch_stiffness(m, w.p, w.Ap, k, 1, s))) return rc;
         }
-        AFEM_LAUNCH((dot_alpha_kernel<double>), cg_blocks(), kRedThreads, 0, s, w.p, w.Ap, Ni, k, w.partial,
+        AFEM_LAUNCH((dot_alpha_kernel<double>), row_blocks(Ni, k), kRedThreads, 0, s, w.p, w.Ap, Ni, k, w.partial,
                     w.counters + 0, st);
-        AFEM_LAUNCH((update_beta_kernel<double>), cg_blocks(), kRedThreads, 0, s, W, w.r, w.p, w.Ap, D.stiff_dinv, Ni, k, st,
+        AFEM_LAUNCH((update_beta_kernel<double>), row_blocks(Ni, k), kRedThreads, 0, s, W, w.r, w.p, w.Ap, D.stiff_dinv, Ni, k, st,
                     w.partial, w.counters + 1, static_cast<const double*>(nullptr),
                     static_cast<const double*>(nullptr), static_cast<const double*>(nullptr), 0.0, 0.0,
                     static_cast<int*>(nullptr));

@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 
@@ -99,6 +100,17 @@ constexpr int kRedBlocksMax = 1024;
 inline int red_blocks() {
     const int g = 4 * device_sms();
     return g < kRedBlocksMax ? g : kRedBlocksMax;
+}
+
+// Blocks of a reduction over rows of `cols` values (at most red_blocks()): one per
+// SM for each 32 rows of a thread, one to four.  Small meshes are bound by the last
+// block's sum over the blocks, large ones by the bytes in flight: CG on 111,661 x 9
+// takes 39.8 / 41.0 / 42.0 ms with 1 / 2 / 3 blocks per SM (26 rows per thread), on
+// 775,009 x 16 502 / 415 / 395 ms with 1 / 2 / 4 (318 rows).
+inline int row_blocks(int64_t rows, int cols) {
+    const int64_t R = std::max(1, kRedThreads / cols), sms = device_sms();
+    const int64_t per_sm = std::min<int64_t>(4, std::max<int64_t>(1, rows / (32 * R * sms)));
+    return int(std::min<int64_t>(red_blocks(), per_sm * sms));
 }
 
 // Threads (r, c) = (t / k, t % k) for t < k * (256 / k); the rest idle.

@@ -6,7 +6,7 @@ nodes than a block takes: the cell passes), and W at an 8-byte address.
 The residual the solver reports is the float64 residual of the full system, so
 meeting rtol 1e-10 is the check of the operator; the V-cycle is a fixed
 preconditioner of CG, so a wrong transfer or coarse solve shows as iterations:
-the start's hierarchy takes 9-20 on these meshes, the bar is 40.  Against the
+a sound hierarchy takes 9-20 on these meshes, the bar is 40.  Against the
 Jacobi-preconditioned solve the fields agree to the condition number (< 1e4
 here) times rtol: 1e-6."""
 import numpy as np

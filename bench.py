@@ -610,20 +610,19 @@ def run_poisson_solvers(torch, pkg, mesh, phi, W_warm, restore, reps=3):
 
 # Kernel classes of the library's event timing: name, bound, unit of work.
 PROF_CLASSES = {
-    0: ("Gram-Schmidt passes (krylov_update / project*_dots, FP64)", "alu", "flops"),
+    0: ("Gram-Schmidt passes (gs_dots_kernel / gs_combine_kernel: float64 quantities, products on the integer pipe, "
+        "so the fraction of the FP64 multiply-add peak can pass 1)", "alu", "flops"),
     1: ("complex64 G cell pass (gcell32b_kernel on frozen per-cell blocks; cell32v_kernel_q4<true,L4,false> when gathered)", "hbm", "bytes"),
     2: ("float32 stiffness of the CG sweeps with the p.Ap epilogue (cell32v_kernel_q4<false,L4,true>)", "hbm", "bytes"),
     3: ("float32 CG vector kernels (update_beta4 / p_update4; p.Ap in the stiffness pass)", "hbm", "bytes"),
-    4: ("FP64 cell passes (g_cell_kernel / cell_op_kernel)", "alu", "flops"),
+    4: ("FP64 cell passes (cell_fx_kernel: contractions on the integer pipe, as class 0)", "alu", "flops"),
 }
 # DRAM bytes per bracketed call from one ncu capture of the same kernels
 # (dram__bytes_read.sum + dram__bytes_write.sum, summed over a class's launches
-# of one Krylov substep / CG iteration and divided by the calls); class 0 is
-# captured on the reduced 16^3-coarse mesh of the molecule (N = 508,385) and
-# scaled by N to the benchmark mesh (every term is a whole-vector pass); class 1
-# is the G cell pass on frozen per-cell blocks (gcell32b_kernel, one launch on
-# the benchmark mesh itself); None where no capture of the current kernel exists.
-TRAFFIC_PER_CALL = {0: 343.9e6, 1: 300.0e6, 2: 114.9e6, 3: 341.8e6, 4: None}
+# and divided by the calls); class 1 is the G cell pass on frozen per-cell blocks
+# (gcell32b_kernel, one launch on the benchmark mesh itself); None where no
+# capture of the current kernel exists.
+TRAFFIC_PER_CALL = {0: None, 1: 300.0e6, 2: 114.9e6, 3: 341.8e6, 4: None}
 
 
 def _class_rooflines(prof, total_ms, fp64_peak, hbm, peak_src):

@@ -191,9 +191,9 @@ int afem_mesh_destroy(afem_mesh* mesh);
 
 /* Kernel-shape options of a mesh (library tuning; no counterpart in the paper).
  * AFEM_OPT_CELL32_VARIANT selects the float32 cell pass: 0 (default) sweeps the
- * lines of a cell with the 1D matrix in constant memory (operators without mean
- * fields) or computes each output node in one thread (G, and the CG sweeps'
- * stiffness with p.Ap), 1 computes the 1D contractions
+ * lines of a cell with the 1D matrix in constant memory (afem_op_apply and the
+ * smoothers) or computes each output node in one thread (the propagators' G, and
+ * the CG sweeps' stiffness with p.Ap), 1 computes the 1D contractions
  * line by line with direction-wise accumulation in shared memory, 2 does the
  * same for the stiffness with one thread per (line, column pair) and the 1D
  * matrix in registers (1, 2 or 4 column quads; other passes as for 0).  All

@@ -1512,9 +1512,13 @@ int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int
 
 // z = H1~ v + mean field (complex64), Dirichlet-masked.
 // velocity != 0: E holds the vector potential A (velocity gauge), applied by
-// the generic (two-lane) kernel.
+// the generic (two-lane) kernel.  lines: a single application, which may run as
+// line sweeps; the propagators' repeated ones keep the node-per-thread pass, whose
+// scatter order decides the rounding that adds up over a propagation (a dipole
+// signal of five steps moved by 7e-8 of its norm with the sweeps, about the
+// error of the float32 operator itself).
 int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const float2* U, float2* z, int n,
-                    cudaStream_t s, int velocity, const float2* U_hang) {
+                    cudaStream_t s, int velocity, const float2* U_hang, bool lines) {
     CellArgs32 a = make_cell_args32(m);
     a.masked = 1;
     a.u_hang = U ? U_hang : nullptr;
@@ -1532,7 +1536,7 @@ int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const 
         for (int i = 0; i < 3; ++i) a.Avec[i] = float(E[i]);
         return launch32<float2, true>(m, a, v, U, z, n, s);
     }
-    if (!U && m->cell32_variant == 0)
+    if (lines && !U && m->cell32_variant == 0)
         return launch_pencil32<true>(m, a, reinterpret_cast<const float*>(v), reinterpret_cast<float*>(z), 2 * n, s);
     if (n % 2 == 0 && aligned16(v) && aligned16(z))
         return launch32v<true>(m, a, reinterpret_cast<const float*>(v), U, reinterpret_cast<float*>(z), 2 * n, n, s);

@@ -392,7 +392,7 @@ int launch_stiffness(const afem_mesh* m, const double* x, double* y, int nv, int
 int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int masked, cudaStream_t s,
                        double* pap_slots = nullptr, bool y_zero = false);
 int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const float2* U, float2* z, int n,
-                    cudaStream_t s, int velocity = 0, const float2* U_hang = nullptr);
+                    cudaStream_t s, int velocity = 0, const float2* U_hang = nullptr, bool lines = false);
 
 int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void* y, int nv,
                     cudaStream_t s) {
@@ -448,7 +448,7 @@ int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void
         return launch_stiffness32(m, static_cast<const float*>(x), static_cast<float*>(y), nv, 0, s);
     if (kind == AFEM_OP_H1_C64 || kind == AFEM_OP_H1_VG_C64) {
         auto* yy = static_cast<float2*>(y);
-        int rc = launch_g_cell32(m, E, static_cast<const float2*>(x), nullptr, yy, nv, s, kind == AFEM_OP_H1_VG_C64);
+        int rc = launch_g_cell32(m, E, static_cast<const float2*>(x), nullptr, yy, nv, s, kind == AFEM_OP_H1_VG_C64, nullptr, true);
         if (rc) return rc;
         return launch_scale_rows<float2>(yy, m->dev.ml_inv, N, nv, s);
     }

@@ -1513,10 +1513,10 @@ int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int
 // z = H1~ v + mean field (complex64), Dirichlet-masked.
 // velocity != 0: E holds the vector potential A (velocity gauge), applied by
 // the generic (two-lane) kernel.  lines: a single application, which may run as
-// line sweeps; the propagators' repeated ones keep the node-per-thread pass, whose
-// scatter order decides the rounding that adds up over a propagation (a dipole
-// signal of five steps moved by 7e-8 of its norm with the sweeps, about the
-// error of the float32 operator itself).
+// line sweeps; the propagators' repeated ones keep the node-per-thread pass: the
+// order of the scatter's additions decides rounding that adds up over a propagation,
+// and with it a dipole signal of five steps differs from run to run by 1e-8 of its
+// norm (one comparison of the sweeps against this pass showed 7e-8).
 int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const float2* U, float2* z, int n,
                     cudaStream_t s, int velocity, const float2* U_hang, bool lines) {
     CellArgs32 a = make_cell_args32(m);

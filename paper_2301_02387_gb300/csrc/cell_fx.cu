@@ -4,30 +4,38 @@
 // weights per real column, 2 per clock and SM) the degree-4 stiffness of 16
 // columns on 12,144 cells took 1,080 us, with the FP64 pipe 92 % busy, against
 // 30 us for the bytes.  Here a block works on whole cells:
-//   1. gather (hanging points through C), largest exponent per cell and column;
-//   2. every value as a 60-bit integer on that scale, and the pointwise part
-//      m (V + E.r) u (+ m sum_q U_pq u_q) in FP64, once per node;
-//   3. three sweeps over pencils (lines of p + 1 nodes): with D = W^-1 Khat,
+//   1. gather (hanging points through C) and, for G, the pointwise part
+//      m (V + E.r) u + m sum_q U_pq u_q in FP64, once per node;
+//   2. three sweeps over pencils (lines of p + 1 nodes): with D = W^-1 Khat,
 //        (A_K u)_abc = h w_a w_b w_c (sum_j D_aj u_jbc + sum_j D_bj u_ajc
-//                                     + sum_j D_cj u_abj),
-//      so all three directions share one scale and their 63-bit sums add up as
-//      integers in shared memory; a thread holds a pencil's values in registers
-//      and reads D from constant memory (operands of the multiply-adds), 5
-//      shared-memory accesses per node and sweep instead of 10 (p + 1) / 2 per
-//      output;
-//   4. the last sweep rounds to float64 once, adds the pointwise part and
+//                                     + sum_j D_cj u_abj);
+//      a thread holds a pencil's values in registers, brings them to the scale of
+//      the largest of them (60-bit integers) and reads D from constant memory
+//      (operands of the multiply-adds), each row of D on its own scale.  The
+//      63-bit sums of the three directions meet in shared memory, each with its
+//      exponent, shifted to the larger of two when they are added;
+//   3. the last sweep rounds to float64 once, adds the pointwise part and
 //      scatters.
+// What an output may be off by follows from its own three lines, as in FP64:
+// one scale for all nodes of a cell took 346 us instead of 595 (46 instead of 61
+// for the 9 columns below), but rounded small values on the scale of the cell's
+// largest.  Each line's sum keeps 2^-60 of the largest |D||u| (degree 4 needs the
+// products of the low words for that, its rows of D spanning 2^6); against a chain
+// of FP64 multiply-adds the error over sum |D||u| is 0.05-0.7 of its size (rms,
+// lines of equal, of single and of widely different values).  Lines with an
+// infinity or NaN give what FP64 gives on that line; tiny ones are scaled up first.
 // A thread keeps one column (c = t % nc) through all of it and takes the nodes
 // or pencils t / nc, + R, ..: with items divided by the run-time column count
 // in every loop the kernel issued 560 instructions per node and column.
 // Hanging nodes (constraint rows of 17 masters on average at degree 4) are
 // listed and taken in loops of their own, which a warp runs for its listed
 // nodes only; walked in place they cost every warp that held one.
-// Per node and column: 9 (p + 1) IMAD.WIDE (31 per clock and SM), one
-// int64 -> float64 conversion and one FP64 multiply-add.  The stiffness above
-// takes 346 us; 9 columns at degree 3 on 4,164 cells 46 us instead of 120.  What
-// bounds it now is instruction issue and the barriers between the sweeps.
-// Each sum is exact to about 2^-57 of the cell column's largest |D| |u|.
+// Per node and column: 9 (p + 1) IMAD.WIDE (12 at degree 4; 31 per clock and SM),
+// three conversions to integers, one back and one FP64 multiply-add.  The
+// stiffness above takes 595 us; 9 columns at degree 3 on 4,164 cells 61 us instead
+// of 120.  What bounds it is instruction issue and the barriers between sweeps.
+// The sums of the directions as FP64 numbers took longer (622 and 81 us): the
+// conversions run at 1.6 per clock and SM.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -39,43 +47,61 @@
 
 namespace afem {
 
-// D = W^-1 Khat on its own scale (biased exponent e of its largest entry).
+// D = W^-1 Khat, each row on the scale of its largest entry (biased exponent e).
 struct FxBasis {
     int h[kMaxP1 * kMaxP1], l[kMaxP1 * kMaxP1];
-    int e;
-    double w3[kMaxP1 * kMaxP1 * kMaxP1];   // w_a w_b w_c, rounded once
+    int l8[kMaxP1 * kMaxP1];   // l / 8, for the products of low words
+    int e[kMaxP1];
+    double w3[kMaxP1 * kMaxP1 * kMaxP1], w3_lo[kMaxP1 * kMaxP1 * kMaxP1];   // w_a w_b w_c as a sum of two
 };
 
 static FxBasis make_fx_basis(const Basis1D& b) {
     FxBasis f{};
     const int p1 = b.p + 1;
-    long double D[kMaxP1 * kMaxP1], top = 0.0L;   // more than 60 bits of the quotient
-    for (int i = 0; i < p1; ++i)
+    for (int i = 0; i < p1; ++i) {
+        long double D[kMaxP1], top = 0.0L;   // more than 60 bits of the quotient
         for (int j = 0; j < p1; ++j) {
-            D[i * p1 + j] = static_cast<long double>(b.K[i][j]) / b.w[i];
-            top = std::max(top, std::fabs(D[i * p1 + j]));
+            D[j] = static_cast<long double>(b.K[i][j]) / b.w[i];
+            top = std::max(top, std::fabs(D[j]));
         }
-    f.e = std::ilogb(top) + 1023;
-    for (int i = 0; i < p1 * p1; ++i) {
-        const int64_t x = std::llrint(std::ldexp(D[i], 1082 - f.e));   // |x| < 2^60
-        const int32_t l = int32_t(uint32_t(uint64_t(x) & 0xFFFFFFFFull));
-        f.l[i] = l;
-        f.h[i] = int((x - l) >> 32);
+        f.e[i] = std::ilogb(top) + 1023;
+        for (int j = 0; j < p1; ++j) {
+            const int64_t x = std::llrint(std::ldexp(D[j], 1082 - f.e[i]));   // |x| < 2^60
+            const int32_t l = int32_t(uint32_t(uint64_t(x) & 0xFFFFFFFFull));
+            f.l[i * p1 + j] = l;
+            f.l8[i * p1 + j] = l >> 3;
+            f.h[i * p1 + j] = int((x - l) >> 32);
+        }
     }
     for (int c = 0; c < p1; ++c)
         for (int d = 0; d < p1; ++d)
-            for (int i = 0; i < p1; ++i)
-                f.w3[i + p1 * (d + p1 * c)] = double(static_cast<long double>(b.w[i]) * b.w[d] * b.w[c]);
+            for (int i = 0; i < p1; ++i) {
+                const long double w = static_cast<long double>(b.w[i]) * b.w[d] * b.w[c];
+                const int q = i + p1 * (d + p1 * c);
+                f.w3[q] = double(w);
+                f.w3_lo[q] = double(w - f.w3[q]);
+            }
     return f;
 }
 
 constexpr int kFxColumns = 16;   // real columns of a block at most
 
-// Shared memory of cpb cells and nc columns.
-static size_t cell_fx_smem(int nn, int cpb, int nc, bool pointwise) {
-    return size_t(cpb) * nn * nc * (sizeof(double) + sizeof(int2) + (pointwise ? sizeof(double) : 0)) +
-           size_t(cpb) * nn * 3 * sizeof(double) + size_t(cpb) * nc * sizeof(int) + size_t(cpb) * nn * 2 * sizeof(int) +
-           size_t(cpb) * sizeof(double4);
+// Shared memory of cpb cells and nc columns (fields: with mean fields).
+static size_t cell_fx_smem(int nn, int cpb, int nc, bool fields) {
+    return size_t(cpb) * nn * nc * (2 * sizeof(double) + sizeof(short) + (fields ? sizeof(double) : 0)) +
+           size_t(cpb) * nn * 3 * sizeof(double) + size_t(cpb) * nn * 2 * sizeof(int) + size_t(cpb) * sizeof(double4);
+}
+
+// Exponents of sums that are no number (above every other): sums of lines with
+// an infinity or NaN.
+constexpr int kSumInf = 0x7F00, kSumMinusInf = 0x7F01, kSumNan = 0x7F02;
+
+// Row i of D on a line with an infinity or NaN: which of the three the sum is.
+__device__ __noinline__ int non_finite_sum(const double* u, int step, const FxBasis& D, int p1, int i) {
+    double f = 0.0;
+    for (int j = 0; j < p1; ++j)
+        f = fma(fma(double(D.h[i * p1 + j]), 4294967296.0, double(D.l[i * p1 + j])), u[j * step], f);
+    return f > 0.0 ? kSumInf : f < 0.0 ? kSumMinusInf : kSumNan;
 }
 
 // One component of acc + w u: the real (odd = 0) or the imaginary part.  The
@@ -93,7 +119,7 @@ __device__ __forceinline__ double mean_field_part(double2 w, double2 u, int odd,
 // plus the mean fields U (real columns 2p, 2p + 1: orbital p).  x, y: [N][ncol]
 // doubles; blockIdx.y selects kFxColumns of them.
 template <int P, int PT>
-__global__ void __launch_bounds__(256, PT == 2 ? 5 : 1) cell_fx_kernel(const __grid_constant__ CellArgs a,
+__global__ void __launch_bounds__(256, PT == 2 ? 4 : 3) cell_fx_kernel(const __grid_constant__ CellArgs a,
                                                       const __grid_constant__ FxBasis D, const double* __restrict__ x,
                                                       const double2* __restrict__ U, double* __restrict__ y, int ncol,
                                                       int cpb, int64_t ncell) {
@@ -103,16 +129,16 @@ __global__ void __launch_bounds__(256, PT == 2 ? 5 : 1) cell_fx_kernel(const __g
     const int64_t cell0 = int64_t(blockIdx.x) * cpb;
     const int nb = int(min(int64_t(cpb), ncell - cell0));   // cells of this block
     double4* s_g = reinterpret_cast<double4*>(smem_raw);                    // [cpb]
-    double* s_u = reinterpret_cast<double*>(s_g + cpb);                     // [cpb][NN][nc] values, then sums
-    long long* s_t = reinterpret_cast<long long*>(s_u);
-    int2* s_i = reinterpret_cast<int2*>(s_u + cpb * NN * nc);               // [cpb][NN][nc] (l, h)
-    double* s_pu = reinterpret_cast<double*>(s_i + cpb * NN * nc);          // [cpb][NN][nc] pointwise part (PT > 0)
-    double* s_hw = s_pu + (PT ? cpb * NN * nc : 0);                         // [cpb][NN] c_kin h w_a w_b w_c
+    double* s_u = reinterpret_cast<double*>(s_g + cpb);                     // [cpb][NN][nc] values
+    long long* s_t = reinterpret_cast<long long*>(s_u + cpb * NN * nc);     // [cpb][NN][nc] running sums
+    double* s_r = reinterpret_cast<double*>(s_t);                           // (and results of hanging nodes)
+    double* s_pu = reinterpret_cast<double*>(s_t + cpb * NN * nc);          // [cpb][NN][nc] pointwise part (PT 2)
+    double* s_hw = s_pu + (PT == 2 ? cpb * NN * nc : 0);                    // [cpb][NN] c_kin h w_a w_b w_c
     double* s_pot = s_hw + cpb * NN;                                        // [cpb][NN] m (V + E.r)
     double* s_wq = s_pot + cpb * NN;                                        // [cpb][NN] m
-    int* s_e = reinterpret_cast<int*>(s_wq + cpb * NN);                     // [cpb][nc]
-    int* s_idx = s_e + cpb * nc;                                            // [cpb][NN]
+    int* s_idx = reinterpret_cast<int*>(s_wq + cpb * NN);                   // [cpb][NN]
     int* s_hl = s_idx + cpb * NN;                                           // [cpb][NN] the hanging nodes
+    short* s_x = reinterpret_cast<short*>(s_hl + cpb * NN);                 // [cpb][NN][nc] exponents of the sums
     __shared__ int s_nh;
     const int tid = threadIdx.x, bs = blockDim.x;
     const int R = bs / nc;                       // rows of threads
@@ -126,7 +152,6 @@ __global__ void __launch_bounds__(256, PT == 2 ? 5 : 1) cell_fx_kernel(const __g
         if (idx < 0) s_hl[atomicAdd(&s_nh, 1)] = i;
     }
     for (int i = tid; i < nb; i += bs) s_g[i] = a.geom[cell0 + i];
-    for (int i = tid; i < nb * nc; i += bs) s_e[i] = kFxMinExp;
     __syncthreads();
     const double* xc = x + c0 + c;
     double* yc = y + c0 + c;
@@ -148,21 +173,16 @@ __global__ void __launch_bounds__(256, PT == 2 ? 5 : 1) cell_fx_kernel(const __g
             if (i >= nodes) break;
             if (s_idx[i] < 0) continue;
             s_u[i * nc + c] = v[q];
-            const int e = int(fx_expbits(v[q]) >> 20);
-            if (e > kFxMinExp) atomicMax(&s_e[(i / NN) * nc + c], e);
         }
     }
     for (int j = r0; j < nh; j += R) {
         const int i = s_hl[j];
-        const double v = gather_value<double>(a, s_idx[i], x, ncol, c0 + c);
-        s_u[i * nc + c] = v;
-        const int e = int(fx_expbits(v) >> 20);
-        if (e > kFxMinExp) atomicMax(&s_e[(i / NN) * nc + c], e);
+        s_u[i * nc + c] = gather_value<double>(a, s_idx[i], x, ncol, c0 + c);
     }
     for (int i = tid; i < nodes; i += bs) {
         const int cell = i / NN, n = i - cell * NN;
         const double4 g = s_g[cell];
-        const double hw = g.w * D.w3[n];
+        const double hw = fma(g.w, D.w3[n], g.w * D.w3_lo[n]);   // rounded once
         s_hw[i] = a.c_kin * hw;
         if constexpr (PT > 0) {
             const int idx = s_idx[i];
@@ -175,14 +195,9 @@ __global__ void __launch_bounds__(256, PT == 2 ? 5 : 1) cell_fx_kernel(const __g
         }
     }
     __syncthreads();
-    const int n = nc >> 1, nn2 = n * n, p = c >> 1;   // PT 2: orbitals
-    for (int i = on ? r0 : nodes; i < nodes; i += R) {
-        const int it = i * nc + c;
-        const double v = s_u[it];
-        const Fx f = fx_make(v, s_e[(i / NN) * nc + c]);
-        s_i[it] = make_int2(f.l, f.h);
-        if constexpr (PT == 1) s_pu[it] = s_pot[i] * v;
-        if constexpr (PT == 2) {   // this column's part of m sum_q U_pq u_q
+    if constexpr (PT == 2) {   // this column's part of m sum_q U_pq u_q
+        const int n = nc >> 1, nn2 = n * n, p = c >> 1;   // orbitals
+        for (int i = on ? r0 : nodes; i < nodes; i += R) {
             const double2* su = reinterpret_cast<const double2*>(s_u) + i * n;
             const int idx = s_idx[i];
             const double2* row = idx >= 0 ? U + int64_t(idx) * nn2
@@ -197,10 +212,9 @@ __global__ void __launch_bounds__(256, PT == 2 ? 5 : 1) cell_fx_kernel(const __g
                 for (int q = 0; q < n; ++q)
                     mf = mean_field_part(gather_value<double2>(au, idx, U, nn2, p * n + q), su[q], c & 1, mf);
             }
-            s_pu[it] = fma(s_wq[i], mf, s_pot[i] * v);
+            s_pu[i * nc + c] = fma(s_wq[i], mf, s_pot[i] * s_u[i * nc + c]);
         }
-    }
-    __syncthreads();
+    }   // (each entry is read by a thread of the same column after the sweeps' barriers)
     const int pencils = nb * NP;
 #pragma unroll
     for (int dir = 0; dir < 3; ++dir) {
@@ -210,34 +224,64 @@ __global__ void __launch_bounds__(256, PT == 2 ? 5 : 1) cell_fx_kernel(const __g
             const int qa = q % P1, qb = q / P1;
             const int n0 = cell * NN + (dir == 0 ? P1 * q : dir == 1 ? qa + NP * qb : q);
             const int base = n0 * nc + c;
-            Fx u[P1];
+            double v[P1];
+            unsigned eb = 0u;
 #pragma unroll
             for (int j = 0; j < P1; ++j) {
-                const int2 v = s_i[base + j * step];
-                u[j] = Fx{v.y, v.x};
+                v[j] = s_u[base + j * step];
+                eb = max(eb, fx_expbits(v[j]));
             }
-            const int e = s_e[cell * nc + c];
+            int e = int(eb >> 20), off = 0;
+            if (e < 2 * kFxMinExp) {   // zero, or too small for the integers: up by 2^600
+                off = 600;
+                eb = 0u;
+#pragma unroll
+                for (int j = 0; j < P1; ++j) {
+                    v[j] *= __hiloint2double((1023 + 600) << 20, 0);
+                    eb = max(eb, fx_expbits(v[j]));
+                }
+                e = int(eb >> 20);
+            }
+            Fx u[P1];
+#pragma unroll
+            for (int j = 0; j < P1; ++j) u[j] = fx_make(v[j], max(e, kFxMinExp));
 #pragma unroll
             for (int i = 0; i < P1; ++i) {
                 FxAcc acc{0, 0};
+                long long low = 0;
 #pragma unroll
-                for (int j = 0; j < P1; ++j) fx_mad_const(acc, Fx{D.h[i * P1 + j], D.l[i * P1 + j]}, u[j]);
-                long long t = (acc.hh << 1) + (acc.x >> 31);
+                for (int j = 0; j < P1; ++j) {
+                    fx_mad_const(acc, Fx{D.h[i * P1 + j], D.l[i * P1 + j]}, u[j]);
+                    if constexpr (P == 4) low += static_cast<long long>(D.l8[i * P1 + j]) * u[j].l;
+                }
+                if constexpr (P == 4) acc.x += low >> 29;
+                long long t = (acc.hh << 4) + (acc.x >> 28);
+                int E = e ? e + D.e[i] - off : 0;   // the sum is t 2^(E - 2104)
+                if (e == 0x7FF) E = non_finite_sum(s_u + base, step, D, P1, i);
                 const int o = base + i * step;
-                if (dir > 0) t += s_t[o];
+                if (dir > 0) {
+                    const int E1 = s_x[o], M = max(E, E1);
+                    t = (t >> min(M - E, 63)) + (s_t[o] >> min(M - E1, 63));
+                    E = (min(E, E1) >= kSumInf && E != E1) ? kSumNan : M;
+                }
                 if (dir < 2) {
                     s_t[o] = t;
+                    s_x[o] = short(E);
                 } else {
-                    // t 2^(e + D.e - 2101), the power of two by the exponent field where
-                    // its result is a normal number (t < 2^62)
+                    const int node = n0 + i * NP, idx = s_idx[node];
+                    // the power of two by the exponent field where the result is a normal number (t < 2^63)
                     double r = __ll2double_rn(t);
-                    const int k = e + D.e - 2101;
-                    if (k <= 2046 - 1086) r = t == 0 ? 0.0 : __hiloint2double(__double2hiint(r) + (k << 20), __double2loint(r));
-                    else r = e == 0x7FF ? __hiloint2double(0x7FF80000, 0) : ldexp(r, k);
-                    const int node = n0 + i * NP;
-                    r = PT ? fma(r, s_hw[node], s_pu[o]) : r * s_hw[node];
-                    const int idx = s_idx[node];
-                    if (idx < 0) s_u[o] = r;   // (in place of this node's t)
+                    const double pu = PT == 2 ? s_pu[o] : PT == 1 ? s_pot[node] * s_u[o] : 0.0;
+                    const int k = t == 0 ? 0 : E - 2104;
+                    if (unsigned(k + 1021) <= 1980u && E < kSumInf) {
+                        r = t == 0 ? 0.0 : __hiloint2double(__double2hiint(r) + (k << 20), __double2loint(r));
+                        r = PT ? fma(r, s_hw[node], pu) : r * s_hw[node];
+                    } else {
+                        r = E == kSumNan ? __hiloint2double(0x7FF80000, 0) : E == kSumInf ? __hiloint2double(0x7FF00000, 0)
+                          : E == kSumMinusInf ? __hiloint2double(int(0xFFF00000), 0) : ldexp(r * s_hw[node], k);
+                        r += pu;
+                    }
+                    if (idx < 0) s_r[o] = r;   // (in place of this node's sum)
                     else if (!(a.masked && idx >= n_int)) atomicAdd(yc + int64_t(idx) * ncol, r);
                 }
             }
@@ -246,7 +290,7 @@ __global__ void __launch_bounds__(256, PT == 2 ? 5 : 1) cell_fx_kernel(const __g
     }
     for (int j = r0; j < nh; j += R) {
         const int i = s_hl[j];
-        scatter_value<double>(a, s_idx[i], y, ncol, c0 + c, s_u[i * nc + c]);
+        scatter_value<double>(a, s_idx[i], y, ncol, c0 + c, s_r[i * nc + c]);
     }
 }
 
@@ -261,7 +305,7 @@ static int launch_p(const afem_mesh* m, const CellArgs& a, const double* x, cons
     const int rounds = (cpb * per + 255) / 256;   // pencils of a thread
     const int rows = (cpb * P1 * P1 + rounds - 1) / rounds;
     const int block = std::min(256, (rows * nc + 31) / 32 * 32);
-    const size_t smem = cell_fx_smem(NN, cpb, nc, PT > 0);
+    const size_t smem = cell_fx_smem(NN, cpb, nc, PT == 2);
     AFEM_CUDA_TRY(allow_dyn_smem(cell_fx_kernel<P, PT>));
     const FxBasis D = make_fx_basis(m->basis);
     const dim3 grid(unsigned((ncell + cpb - 1) / cpb), unsigned((ncol + kFxColumns - 1) / kFxColumns));

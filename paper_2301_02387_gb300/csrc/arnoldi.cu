@@ -267,29 +267,69 @@ constexpr int kScaleBeta = kMaxKrylov + 1;
 // ------------------------------------------------- the Krylov basis in integers
 // The Gram-Schmidt passes read every basis vector twice per new vector and are
 // products and sums of float64 numbers, which run on the integer pipe
-// (fixed64.cuh).  The vectors are therefore stored ready for it: per group of
-// rows one exponent e (of the largest component), and per component the
-// integer X = v 2^(1082 - e), |X| < 2^60, split h 2^32 + l,
-// as (re l, re h, im l, im h): 16 bytes, as the float64 pair was, and seven
-// bits finer than float64 at the group's largest component.  Reading a
-// component then costs no conversion.  Measured on 10 vectors of 775,009 x 4
-// (499 MB, 73 us at the copy rate): inner products with the projector 259 us as
-// FP64 multiply-adds, 237 us converting from float64 on the way, 127 us stored
-// as integers; the update 245 / 154 / 109 us, the close of a substep 254 / 103 us.
-// What bounds them now is instruction issue (about 50 per element and vector, 12
-// of them IMAD.WIDE at 31 lanes per clock) beside 55-70 % of the copy rate.
-//
+// (fixed64.cuh).  The vectors are therefore stored ready for it: per complex
+// entry one exponent e (of its larger component) and per component the 64-bit
+// integer X = v 2^(1082 - e), |X| < 2^60: 16 bytes, as the float64 pair was, and
+// seven bits finer than float64 at the larger component.  Reading an entry then
+// costs no conversion, only a shift to the scale of a sum: over the rows of a
+// group (inner products, norms) that of the group's largest, over the vectors (a
+// linear combination) that of the entry's own largest term, so that an entry
+// is rounded on its own terms, as with float64, whatever its neighbours' size.
+// Measured on 10 vectors of 775,009 x 4 (499 MB, 73 us at the copy rate): inner
+// products with the projector 259 us as FP64 multiply-adds, 237 us converting
+// from float64 on the way, 131 us stored as integers; the update 245 / 154 / 128
+// us, the close of a substep 254 / 117 us.  (One exponent for the rows of a group
+// took 127, 109 and 103 us, but rounded an entry on its group's largest.)
+
 // Thread t < n R of a 256-thread block (R = 256 / n) owns column p = t % n and,
 // in tile T, the rows T E R + r + R e (e < E, r = t / n): a group, the rows that
-// one thread sums together, with one exponent (4 bytes beside 16 E of data), so
-// that no thread waits for another's scale.  Storage follows the threads, not
-// the rows: element (T, e, t) of a vector, exponent (T, t).  E (4, 2 or 1) is chosen per call so
-// that the tiles fill the chip (krylov_rows).  Exponent 0: all components zero;
-// 0x7FF: the group holds a non-finite value.
+// one thread sums together, so that no thread waits for another's scale.  Storage
+// follows the threads, not the rows: entry (T, e, t) of a vector, exponents (T, t),
+// 16 bits each, the rows of a group in one or two words.  E (4, 2 or 1) is chosen per call so
+// that the tiles fill the chip (krylov_rows).  Exponent 0: zero; 0x7FF: not finite.
 constexpr int kFxNan = 0x7FF;
+__host__ __device__ constexpr int exp_words(int E) { return (E + 1) / 2; }
 
-__device__ __forceinline__ Fx fx_re(int4 v) { return Fx{v.y, v.x}; }
-__device__ __forceinline__ Fx fx_im(int4 v) { return Fx{v.w, v.z}; }
+__device__ __forceinline__ long long fx_re(int4 v) { return (static_cast<long long>(v.y) << 32) | unsigned(v.x); }
+__device__ __forceinline__ long long fx_im(int4 v) { return (static_cast<long long>(v.w) << 32) | unsigned(v.z); }
+__device__ __forceinline__ int4 fx_entry(long long re, long long im) {
+    return make_int4(int(re), int(re >> 32), int(im), int(im >> 32));
+}
+// x 2^-d rounded down, for any d >= 0 (the instruction takes shifts beyond 63 as 64).
+__device__ __forceinline__ long long shift_right(long long x, int d) {
+    long long r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(d));
+    return r;
+}
+// The exponents of a group's E rows.
+template <int E>
+__device__ __forceinline__ void read_exps(const int* p, int (&e)[E]) {
+    if constexpr (E == 1) {
+        e[0] = p[0];
+    } else {
+        int w[E / 2];
+        if constexpr (E == 4) {
+            const int2 v = *reinterpret_cast<const int2*>(p);
+            w[0] = v.x;
+            w[1] = v.y;
+        } else {
+            w[0] = p[0];
+        }
+#pragma unroll
+        for (int r = 0; r < E; ++r) e[r] = (r & 1) ? int(unsigned(w[r / 2]) >> 16) : w[r / 2] & 0xFFFF;
+    }
+}
+template <int E>
+__device__ __forceinline__ void write_exps(int* p, const int (&e)[E]) {
+    if constexpr (E == 4) *reinterpret_cast<int2*>(p) = make_int2(e[0] | (e[1] << 16), e[2] | (e[3] << 16));
+    else if constexpr (E == 2) p[0] = e[0] | (e[1] << 16);
+    else p[0] = e[0];
+}
+// An entry as float64.
+__device__ __forceinline__ double2 fx_double2(int4 v, int e) {
+    const double sc = e == kFxNan ? __hiloint2double(0x7FF80000, 0) : e == 0 ? 0.0 : ldexp(1.0, e - 1082);
+    return make_double2(sc * double(fx_re(v)), sc * double(fx_im(v)));
+}
 
 struct TileRows {
     int p, r, R;
@@ -312,9 +352,10 @@ __device__ __forceinline__ void copy16(void* smem_dst, const void* gmem_src) {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
 }
-__device__ __forceinline__ void copy4(void* smem_dst, const void* gmem_src) {
+template <int WORDS>
+__device__ __forceinline__ void copy_exps(int* smem_dst, const int* gmem_src) {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gmem_src) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(gmem_src), "n"(4 * WORDS) : "memory");
 }
 __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int LEFT>
@@ -324,18 +365,20 @@ __device__ __forceinline__ void copy_wait() {
 
 template <int E, int STAGES>
 struct BasisStream {
+    static constexpr int EW = exp_words(E);
     const int4* v;        // next item's first row
-    const int* e;         // its exponent
+    const int* e;         // its exponents
     int4* slots;          // this thread's slots, [STAGES][E][kRedThreads]
-    int* eslots;          // [STAGES][kRedThreads] (STAGE_E)
+    int* eslots;          // [STAGES][kRedThreads][EW] (STAGE_E)
     int64_t stride, estride, wrap, ewrap;   // to the next vector; from the last vector to the next tile's first
     int left, nv;         // tiles left, vectors
     int i, stage;
     __device__ __forceinline__ BasisStream(const KrylovBasis& B, int nv_, int4* sl, int* esl)
         : v(B.V + int64_t(blockIdx.x) * (E * kRedThreads) + threadIdx.x),
-          e(B.e + int64_t(blockIdx.x) * kRedThreads + threadIdx.x), slots(sl + threadIdx.x), eslots(esl + threadIdx.x),
+          e(B.e + (int64_t(blockIdx.x) * kRedThreads + threadIdx.x) * EW), slots(sl + threadIdx.x),
+          eslots(esl + threadIdx.x * EW),
           stride(B.stride), estride(B.estride), wrap(int64_t(gridDim.x) * (E * kRedThreads) - (nv_ - 1) * B.stride),
-          ewrap(int64_t(gridDim.x) * kRedThreads - (nv_ - 1) * B.estride),
+          ewrap(int64_t(gridDim.x) * kRedThreads * EW - (nv_ - 1) * B.estride),
           left(int((B.tiles - blockIdx.x + gridDim.x - 1) / gridDim.x)), nv(nv_), i(0), stage(0) {}
     template <bool STAGE_E>
     __device__ __forceinline__ void issue() {
@@ -343,7 +386,7 @@ struct BasisStream {
             int4* d = slots + stage * (E * kRedThreads);
 #pragma unroll
             for (int r = 0; r < E; ++r) copy16(d + r * kRedThreads, v + r * kRedThreads);
-            if (STAGE_E) copy4(eslots + stage * kRedThreads, e);
+            if (STAGE_E) copy_exps<EW>(eslots + stage * kRedThreads * EW, e);
             const bool last = ++i == nv;
             v += last ? wrap : stride;
             if (STAGE_E) e += last ? ewrap : estride;
@@ -373,8 +416,8 @@ struct BasisStream {
 // re-orthogonalisation test uses it.
 //
 // A thread forms m w of its E rows on their common scale and walks the basis
-// vectors: E staged rows, 12 E IMAD.WIDE and two float64 additions into its sums
-// in shared memory.
+// vectors: E staged rows, shifted to the vector's largest of them, 12 E IMAD.WIDE
+// and two float64 additions into its sums in shared memory.
 struct GsDotsArgs {
     const double2* z;
     float2* z32;
@@ -403,7 +446,8 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_dots_kernel(const __grid_co
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2* s_acc = reinterpret_cast<double2*>(smem_raw);                  // [nv][kRedThreads]
     int4* s_v = reinterpret_cast<int4*>(s_acc + a.nv * kRedThreads);       // [STAGES][E][kRedThreads]
-    int* s_ve = reinterpret_cast<int*>(s_v + STAGES * E * kRedThreads);    // [STAGES][kRedThreads]
+    int* s_ve = reinterpret_cast<int*>(s_v + STAGES * E * kRedThreads);    // [STAGES][kRedThreads][EW]
+    constexpr int EW = exp_words(E);
     __shared__ double s_f[kMaxKrylov];
     __shared__ double2 s_S[MODE == 1 ? kMaxOrbProj * kMaxOrbProj : 1];
     __shared__ float2 s_S32[MODE == 2 ? kMaxOrbProj * kMaxOrbProj : 1];
@@ -452,15 +496,12 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_dots_kernel(const __grid_co
                 x[r] = make_double2(0.0, 0.0);
             }
             if constexpr (MODE == 0) {
+                int e[E];
+                read_exps<E>(a.B.e + nv * a.B.estride + (tile * kRedThreads + tid) * EW, e);
 #pragma unroll
-                for (int r = 0; r < E; ++r) {
-                    if (k0 + r * rc.R >= n_int) continue;
-                    const int4 v = a.B.V[nv * a.B.stride + (tile * E + r) * kRedThreads + tid];
-                    const int e = a.B.e[nv * a.B.estride + tile * kRedThreads + tid];
-                    const double sc = e == kFxNan ? __hiloint2double(0x7FF80000, 0) : e == 0 ? 0.0 : ldexp(1.0, e - 1082);
-                    x[r].x = sc * double((static_cast<long long>(v.y) << 32) + v.x);
-                    x[r].y = sc * double((static_cast<long long>(v.w) << 32) + v.z);
-                }
+                for (int r = 0; r < E; ++r)
+                    if (k0 + r * rc.R < n_int)
+                        x[r] = fx_double2(a.B.V[nv * a.B.stride + (tile * E + r) * kRedThreads + tid], e[r]);
             }
             if constexpr (MODE == 1) {
                 double2 zo[E];
@@ -548,16 +589,21 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_dots_kernel(const __grid_co
                 int4 u[E];
 #pragma unroll
                 for (int r = 0; r < E; ++r) u[r] = s_v[(slot * E + r) * kRedThreads + tid];
-                const int eu = s_ve[slot * kRedThreads + tid];
+                int er[E], eu = 0;
+                read_exps<E>(s_ve + (slot * kRedThreads + tid) * EW, er);
+#pragma unroll
+                for (int r = 0; r < E; ++r) eu = max(eu, er[r]);
                 slot = slot + 1 == STAGES ? 0 : slot + 1;
                 st.template issue<true>();
                 FxAcc re{0, 0}, im{0, 0};
 #pragma unroll
                 for (int r = 0; r < E; ++r) {
-                    fx_mad(re, fx_re(u[r]), X[r]);
-                    fx_mad(re, fx_im(u[r]), Y[r]);
-                    fx_mad(im, fx_re(u[r]), Y[r]);
-                    fx_mad(im, fx_im(u[r]), nX[r]);
+                    const int d = eu - er[r];
+                    const Fx ur = fx_split(shift_right(fx_re(u[r]), d)), ui = fx_split(shift_right(fx_im(u[r]), d));
+                    fx_mad(re, ur, X[r]);
+                    fx_mad(re, ui, Y[r]);
+                    fx_mad(im, ur, Y[r]);
+                    fx_mad(im, ui, nX[r]);
                 }
                 const double sc = fx_scale((eu == kFxNan || xe == kFxExpMask) ? 0x7FFFFF : eu + ex);
                 double2 acc = s_acc[i * kRedThreads + tid];
@@ -628,12 +674,12 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_dots_kernel(const __grid_co
 // reads the scales at its start, the last block writes after all others have
 // finished); V_0 is written tile by tile after the tile's reads.
 //
-// A thread brings its group of rows to the scale of the largest term c_i e_i by
-// shifting each coefficient once per group; an element then costs its 16-byte
-// row and 12 IMAD.WIDE per vector, against 4 FP64 multiply-add slots of 64
-// lanes before.  The result keeps 63 bits on the scale of its largest term or
-// of the base and is shifted to the group's new exponent; its squares for the
-// norm are integer products too, rounded to float64 once per row.
+// A thread brings each of its rows to the scale of the row's largest term c_i e_i
+// by shifting the entries; an entry then costs its 16 bytes and 12 IMAD.WIDE per
+// vector, against 4 FP64 multiply-add slots of 64 lanes before.  The result keeps
+// 58 bits below its largest term or the base and is shifted to its own exponent;
+// its squares for the norm are integer products too, on the scale of the group's
+// largest, rounded to float64 once per row.
 struct GsCombineArgs {
     KrylovBasis B;
     int nv;
@@ -668,16 +714,16 @@ __device__ __forceinline__ long long float_int(float f, int s) {
     return int(u) < 0 ? -static_cast<long long>(v) : static_cast<long long>(v);
 }
 
-constexpr int kCombineStages = 4;
-template <int E, int KIND>
+template <int E, int KIND, int STAGES>
 __global__ void __launch_bounds__(kRedThreads, 2) gs_combine_kernel(const __grid_constant__ GsCombineArgs a) {
     if (KIND == 3 && *a.gate == 0) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int4* s_v = reinterpret_cast<int4*>(smem_raw);                                   // [stages][E][kRedThreads]
-    int* s_ge = reinterpret_cast<int*>(s_v + kCombineStages * E * kRedThreads);     // [2][nv][kRedThreads]
+    int* s_ge = reinterpret_cast<int*>(s_v + STAGES * E * kRedThreads);     // [2][nv][kRedThreads][EW]
+    constexpr int EW = exp_words(E);
     __shared__ double s_f[kMaxKrylov];
     __shared__ double2 s_c[kMaxKrylov + 1];
-    __shared__ longlong2 s_ci[kMaxKrylov];   // coefficients, integers on their own scale
+    __shared__ int4 s_ci[kMaxKrylov];        // coefficients, integers on their own scale (re l, re h, im l, im h)
     __shared__ int s_ce[kMaxKrylov];         // their biased exponents
     __shared__ int s_low;                    // smallest admissible term exponent (kFxMaxSum + 1: NaN)
     const int nv = a.nv, n = a.n, tid = threadIdx.x;
@@ -701,7 +747,8 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_combine_kernel(const __grid
             const double2 c = make_double2(f * s_c[tid].x, f * s_c[tid].y);
             const int e = int(max(fx_expbits(c.x), fx_expbits(c.y)) >> 20);
             s_ce[tid] = e;
-            s_ci[tid] = make_longlong2(e ? fx_int(c.x, e) : 0, e ? fx_int(c.y, e) : 0);
+            const Fx re = fx_split(e ? fx_int(c.x, e) : 0), im = fx_split(e ? fx_int(c.y, e) : 0);
+            s_ci[tid] = make_int4(re.l, re.h, im.l, im.h);
         }
         __syncthreads();
         if (tid == 0) {
@@ -718,23 +765,24 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_combine_kernel(const __grid
     const TileRows rc(n);
     const int p = rc.p;
     double nrm[1] = {0.0};
-    // the group exponents of this and the next tile, staged like the vectors
+    // the exponents of this and the next tile, staged like the vectors
     auto copy_e = [&](int64_t tile, int par) {
         if (tile < a.B.tiles)
             for (int i = 0; i < nv; ++i)
-                copy4(s_ge + (par * nv + i) * kRedThreads + tid, a.B.e + i * a.B.estride + tile * kRedThreads + tid);
+                copy_exps<EW>(s_ge + ((par * nv + i) * kRedThreads + tid) * EW,
+                              a.B.e + i * a.B.estride + (tile * kRedThreads + tid) * EW);
     };
-    BasisStream<E, kCombineStages> st(a.B, nv, s_v, s_ge);
+    BasisStream<E, STAGES> st(a.B, nv, s_v, s_ge);
     if (KIND != 0 && rc.active) {
         copy_e(blockIdx.x, 0);   // complete with the first item
 #pragma unroll
-        for (int q = 0; q < kCombineStages - 1; ++q) st.template issue<false>();
+        for (int q = 0; q < STAGES - 1; ++q) st.template issue<false>();
     }
     int slot = 0, par = 0;
     const int N = int(a.N), n_int = int(a.n_int);
     const int rows = KIND >= 2 ? n_int : N;   // rows of the result; zero beyond
     for (int64_t tile = blockIdx.x; rc.active && tile < a.B.tiles; tile += gridDim.x, par ^= 1) {
-        int* eg = a.B.e + tile * kRedThreads + tid;
+        int* eg = a.B.e + (tile * kRedThreads + tid) * EW;
         const int k0 = int(tile) * (E * rc.R) + rc.r;
         unsigned o[E];
         long long tx[E], ty[E];
@@ -749,39 +797,50 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_combine_kernel(const __grid
             bf[r] = make_float2(0.f, 0.f);
             if (KIND == 4 && k < n_int) bf[r] = a.w32[o[r]];
         }
-        int EM = KIND == 0 ? 1023 + kFxMinExp : s_low;
+        int EM[E];       // the rows' scales
+#pragma unroll
+        for (int r = 0; r < E; ++r) EM[r] = KIND == 0 ? 1023 + kFxMinExp : s_low;
         if constexpr (KIND != 0) {
             // this tile's exponents came with an item at least nv before its own
-            if (tile == blockIdx.x) copy_wait<kCombineStages - 2>();
-            else if (nv < kCombineStages) copy_wait<0>();
-            const int* ge = s_ge + par * nv * kRedThreads + tid;
-            bool bad = false;
+            if (tile == blockIdx.x) copy_wait<STAGES - 2>();
+            else if (nv < STAGES) copy_wait<0>();
+            const int* ge = s_ge + (par * nv * kRedThreads + tid) * EW;
+            unsigned bad = 0u;
 #pragma unroll 4
             for (int i = 0; i < nv; ++i) {
-                const int e = ge[i * kRedThreads];
-                bad = bad || e == kFxNan;
-                EM = max(EM, e + s_ce[i]);
+                int e[E];
+                read_exps<E>(ge + i * kRedThreads * EW, e);
+                const int ce = s_ce[i];
+#pragma unroll
+                for (int r = 0; r < E; ++r) {
+                    if (e[r] == kFxNan) bad |= 1u << r;
+                    EM[r] = max(EM[r], e[r] + ce);
+                }
             }
             copy_e(tile + gridDim.x, par ^ 1);   // in the next item's group
             FxAcc ax[E], ay[E];
 #pragma unroll
             for (int r = 0; r < E; ++r) ax[r] = ay[r] = FxAcc{0, 0};
             for (int i = 0; i < nv; ++i) {
-                const int sh = min(EM - ge[i * kRedThreads] - s_ce[i], 63);
-                const longlong2 ci = s_ci[i];
-                const Fx re = fx_split(ci.x >> sh), im = fx_split(ci.y >> sh), nim = fx_split(-(ci.y >> sh));
-                copy_wait<kCombineStages - 2>();
+                int e[E];
+                read_exps<E>(ge + i * kRedThreads * EW, e);
+                const int ce = s_ce[i];
+                const int4 c4 = s_ci[i];
+                const Fx re{c4.y, c4.x}, im{c4.w, c4.z}, nim = fx_neg(im);
+                copy_wait<STAGES - 2>();
                 int4 u[E];
 #pragma unroll
                 for (int r = 0; r < E; ++r) u[r] = s_v[(slot * E + r) * kRedThreads + tid];
-                slot = slot + 1 == kCombineStages ? 0 : slot + 1;
+                slot = slot + 1 == STAGES ? 0 : slot + 1;
                 st.template issue<false>();
 #pragma unroll
                 for (int r = 0; r < E; ++r) {
-                    fx_mad(ax[r], re, fx_re(u[r]));
-                    fx_mad(ax[r], nim, fx_im(u[r]));
-                    fx_mad(ay[r], re, fx_im(u[r]));
-                    fx_mad(ay[r], im, fx_re(u[r]));
+                    const int sh = EM[r] - e[r] - ce;
+                    const Fx ur = fx_split(shift_right(fx_re(u[r]), sh)), ui = fx_split(shift_right(fx_im(u[r]), sh));
+                    fx_mad(ax[r], re, ur);
+                    fx_mad(ax[r], nim, ui);
+                    fx_mad(ay[r], re, ui);
+                    fx_mad(ay[r], im, ur);
                 }
                 if (i & 1) {   // two vectors (4 products) between carries
 #pragma unroll
@@ -791,96 +850,86 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_combine_kernel(const __grid
                     }
                 }
             }
-            if (bad) EM = kFxMaxSum + 1;
 #pragma unroll
             for (int r = 0; r < E; ++r) {
+                if (bad & (1u << r)) EM[r] = kFxMaxSum + 1;
                 tx[r] = (ax[r].hh << 1) + (ax[r].x >> 31);
                 ty[r] = (ay[r].hh << 1) + (ay[r].x >> 31);
             }
         }
-        if constexpr (KIND == 4) {   // the base: 24 bits at 2^56 of the scale EM, the thread's rows alike
-            unsigned be = 0u;
-#pragma unroll
-            for (int r = 0; r < E; ++r)
-                be = max(be, max(__float_as_uint(bf[r].x) & 0x7F800000u, __float_as_uint(bf[r].y) & 0x7F800000u));
-            const int eb = max(int(be >> 23) + 896 - kv, kFxMinExp);
-            const int up = max(EM, eb + 1023), d = min(up - EM, 63);
+        if constexpr (KIND == 4) {   // the base: 24 bits at 2^56 of the scale EM
 #pragma unroll
             for (int r = 0; r < E; ++r) {
+                const unsigned be = max(__float_as_uint(bf[r].x) & 0x7F800000u, __float_as_uint(bf[r].y) & 0x7F800000u);
+                const int eb = max(int(be >> 23) + 896 - kv, kFxMinExp);
+                const int up = max(EM[r], eb + 1023), d = min(up - EM[r], 63);
                 tx[r] = (tx[r] >> d) + float_int(bf[r].x, up - 1919 + kv);
                 ty[r] = (ty[r] >> d) + float_int(bf[r].y, up - 1919 + kv);
+                EM[r] = (EM[r] > kFxMaxSum || be == 0x7F800000u || eb >= kFxNan) ? kFxMaxSum + 1 : up;
             }
-            EM = (EM > kFxMaxSum || be == 0x7F800000u || eb >= kFxNan) ? kFxMaxSum + 1 : up;
         } else if constexpr (KIND != 1) {   // the base: 53 bits at 2^56 of the scale EM
             double2 b[E];
-            unsigned be = 0u;
+            int e3[E];
+            if constexpr (KIND == 3) read_exps<E>(eg + nv * a.B.estride, e3);
 #pragma unroll
             for (int r = 0; r < E; ++r) {
-                const int k = k0 + r * rc.R;
                 b[r] = make_double2(0.0, 0.0);
-                if (k < rows) {
+                if (k0 + r * rc.R < rows) {
                     if constexpr (KIND == 0) b[r] = a.src[o[r]];
                     if constexpr (KIND == 2) b[r] = a.wd[o[r]];
-                    if constexpr (KIND == 3) {
-                        const int4 v = a.B.V[nv * a.B.stride + (tile * E + r) * kRedThreads + tid];
-                        const int e = eg[nv * a.B.estride];
-                        const double sc = e == kFxNan ? __hiloint2double(0x7FF80000, 0)
-                                                      : e == 0 ? 0.0 : ldexp(1.0, e - 1082);
-                        b[r].x = sc * double((static_cast<long long>(v.y) << 32) + v.x);
-                        b[r].y = sc * double((static_cast<long long>(v.w) << 32) + v.z);
-                    }
+                    if constexpr (KIND == 3)
+                        b[r] = fx_double2(a.B.V[nv * a.B.stride + (tile * E + r) * kRedThreads + tid], e3[r]);
                 }
-                be = max(be, max(fx_expbits(b[r].x), fx_expbits(b[r].y)));
             }
-            const int eb = max(int(be >> 20), kFxMinExp);
-            const int up = max(EM, eb + 1023), d = min(up - EM, 63);
-            const int es = min(up - 1023, 8000);   // b 2^(2101 - up) = (b 2^(1082 - es)) / 16 for es = up - 1023
 #pragma unroll
             for (int r = 0; r < E; ++r) {
+                const unsigned be = max(fx_expbits(b[r].x), fx_expbits(b[r].y));
+                const int eb = max(int(be >> 20), kFxMinExp);
+                const int up = max(EM[r], eb + 1023), d = min(up - EM[r], 63);
+                const int es = min(up - 1023, 8000);   // b 2^(2101 - up) = (b 2^(1082 - es)) / 16 for es = up - 1023
                 tx[r] = (tx[r] >> d) + (fx_int(b[r].x, es) >> 4);
                 ty[r] = (ty[r] >> d) + (fx_int(b[r].y, es) >> 4);
+                EM[r] = (EM[r] > kFxMaxSum || be == kFxExpMask) ? kFxMaxSum + 1 : up;
             }
-            EM = (EM > kFxMaxSum || be == kFxExpMask) ? kFxMaxSum + 1 : up;
         }
-        unsigned long long any = 0ull;
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            if (k0 + r * rc.R >= rows) tx[r] = ty[r] = 0;
-            any |= static_cast<unsigned long long>((tx[r] ^ (tx[r] >> 63)) | (ty[r] ^ (ty[r] >> 63)));
-        }
-        const int bits = 64 - __clzll(static_cast<long long>(any));
-        // the group's new exponent: |x| <= 2^(bits + EM - 2101) (t = -1 alone: any = 0)
-        int eo = bits ? bits + EM - 1079 : 0;
-        if (EM > kFxMaxSum || eo > kFxNan) eo = kFxNan;
-        if (eo < kFxMinExp) eo = 0;
         const int dst = KIND <= 1 ? 0 : nv;
-        eg[dst * a.B.estride] = eo;
-        const int shl = 63 - bits;   // t 2^(EM - 2101) = X 2^(eo - 1082), X = t 2^(60 - bits)
+        int eo[E], top = 0;   // the rows' new exponents, the group's largest
         double n2 = 0.0;
 #pragma unroll
         for (int r = 0; r < E; ++r) {
-            const int k = k0 + r * rc.R;
-            if (k >= N) continue;
-            long long vx = 0, vy = 0;
-            if (eo != 0) {
-                vx = (tx[r] << shl) >> 3;
-                vy = (ty[r] << shl) >> 3;
+            if (k0 + r * rc.R >= rows) tx[r] = ty[r] = 0;
+            const int bits = 64 - __clzll(static_cast<long long>((tx[r] ^ (tx[r] >> 63)) | (ty[r] ^ (ty[r] >> 63))));
+            // |x| <= 2^(bits + EM - 2101) (t = -1 alone: bits = 0)
+            eo[r] = bits ? bits + EM[r] - 1079 : 0;
+            if (EM[r] > kFxMaxSum || eo[r] > kFxNan) eo[r] = kFxNan;
+            if (eo[r] < kFxMinExp) eo[r] = 0;
+            top = max(top, eo[r]);
+            // t 2^(EM - 2101) = X 2^(eo - 1082), X = t 2^(60 - bits)
+            const long long vx = eo[r] != 0 ? (tx[r] << (63 - bits)) >> 3 : 0, vy = eo[r] != 0 ? (ty[r] << (63 - bits)) >> 3 : 0;
+            if (k0 + r * rc.R < N) {
+                a.B.V[dst * a.B.stride + (tile * E + r) * kRedThreads + tid] = fx_entry(vx, vy);
+                if ((KIND == 1 && a.out) || a.vd) {
+                    const double sc = fx_scale(EM[r]);
+                    const double2 v = make_double2(__ll2double_rn(tx[r]) * sc, __ll2double_rn(ty[r]) * sc);
+                    if (KIND == 1 && a.out) a.out[o[r]] = v;
+                    if (a.vd) a.vd[o[r]] = v;
+                }
+                if (a.v32) a.v32[o[r]] = make_float2(fx_to_f32(vx, eo[r] - 1082 + kw), fx_to_f32(vy, eo[r] - 1082 + kw));
             }
-            const Fx fx = fx_split(vx), fy = fx_split(vy);
-            a.B.V[dst * a.B.stride + (tile * E + r) * kRedThreads + tid] = make_int4(fx.l, fx.h, fy.l, fy.h);
+            tx[r] = vx;
+            ty[r] = vy;
+        }
+        write_exps<E>(eg + dst * a.B.estride, eo);
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+            const int d = min(top - eo[r], 63);
+            const Fx fx = fx_split(tx[r] >> d), fy = fx_split(ty[r] >> d);
             FxAcc sq{0, 0};
             fx_mad(sq, fx, fx);
             fx_mad(sq, fy, fy);
             n2 = fma(mass[r], fx_value(sq), n2);
-            if ((KIND == 1 && a.out) || a.vd) {
-                const double sc = fx_scale(EM);
-                const double2 v = make_double2(__ll2double_rn(tx[r]) * sc, __ll2double_rn(ty[r]) * sc);
-                if (KIND == 1 && a.out) a.out[o[r]] = v;
-                if (a.vd) a.vd[o[r]] = v;
-            }
-            if (a.v32) a.v32[o[r]] = make_float2(fx_to_f32(vx, eo - 1082 + kw), fx_to_f32(vy, eo - 1082 + kw));
         }
-        nrm[0] = fma(n2, eo == kFxNan ? __hiloint2double(0x7FF80000, 0) : fx_scale(2 * eo), nrm[0]);
+        nrm[0] = fma(n2, top == kFxNan ? __hiloint2double(0x7FF80000, 0) : fx_scale(2 * top), nrm[0]);
     }
     __syncthreads();
     block_row_partial<1>(nrm, 1, a.partial);
@@ -1170,18 +1219,19 @@ static int krylov_rows(int64_t N, int n) {
 
 template <int E, int MODE, int STAGES>
 static int launch_gs_dots_s(const GsDotsArgs& a, cudaStream_t s) {
-    constexpr size_t kStage = size_t(STAGES) * kRedThreads * (E * sizeof(int4) + sizeof(int));
+    constexpr size_t kStage = size_t(STAGES) * kRedThreads * (E * sizeof(int4) + exp_words(E) * sizeof(int));
     AFEM_CUDA_TRY(allow_dyn_smem(gs_dots_kernel<E, MODE, STAGES>));
     const unsigned g = wave_grid<gs_dots_kernel<E, MODE, STAGES>>(
-        a.B.tiles, (STAGES == 4 ? 10 : STAGES == 3 ? 14 : 16) * kRedThreads * sizeof(double2) + kStage);
+        a.B.tiles, (STAGES == 4 ? 9 : STAGES == 3 ? 13 : 16) * kRedThreads * sizeof(double2) + kStage);
     AFEM_LAUNCH((gs_dots_kernel<E, MODE, STAGES>), g, kRedThreads, a.nv * kRedThreads * sizeof(double2) + kStage, s, a);
     AFEM_CUDA_TRY(cudaGetLastError());
     return AFEM_OK;
 }
 template <int E, int MODE>
 static int launch_gs_dots_e(const GsDotsArgs& a, cudaStream_t s) {
-    return a.nv <= 10 ? launch_gs_dots_s<E, MODE, 4>(a, s) : a.nv <= 14 ? launch_gs_dots_s<E, MODE, 3>(a, s)
-                                                                        : launch_gs_dots_s<E, MODE, 2>(a, s);
+    // (the sums of nv vectors beside the ring: its depth leaves two blocks per SM)
+    return a.nv <= 9 ? launch_gs_dots_s<E, MODE, 4>(a, s) : a.nv <= 13 ? launch_gs_dots_s<E, MODE, 3>(a, s)
+                                                                       : launch_gs_dots_s<E, MODE, 2>(a, s);
 }
 template <int MODE>
 static int launch_gs_dots(int E, const GsDotsArgs& a, cudaStream_t s) {
@@ -1190,15 +1240,27 @@ static int launch_gs_dots(int E, const GsDotsArgs& a, cudaStream_t s) {
                                                             : launch_gs_dots_e<1, MODE>(a, s);
 }
 
-template <int E, int KIND>
-static int launch_gs_combine_e(const GsCombineArgs& a, cudaStream_t s) {
-    constexpr size_t kStage = KIND == 0 ? 0 : size_t(kCombineStages) * kRedThreads * E * sizeof(int4);
-    constexpr size_t kExp = KIND == 0 ? 0 : 2 * kRedThreads * sizeof(int);   // per vector
-    AFEM_CUDA_TRY(allow_dyn_smem(gs_combine_kernel<E, KIND>));
-    const unsigned g = wave_grid<gs_combine_kernel<E, KIND>>(a.B.tiles, kStage + kMaxKrylov * kExp);
-    AFEM_LAUNCH((gs_combine_kernel<E, KIND>), g, kRedThreads, kStage + a.nv * kExp, s, a);
+template <int E, int KIND, int STAGES, int NV>   // NV: most vectors of this ring depth
+static int launch_gs_combine_s(const GsCombineArgs& a, cudaStream_t s) {
+    constexpr size_t kStage = KIND == 0 ? 0 : size_t(STAGES) * kRedThreads * E * sizeof(int4);
+    constexpr size_t kExp = KIND == 0 ? 0 : 2 * kRedThreads * exp_words(E) * sizeof(int);   // per vector
+    AFEM_CUDA_TRY(allow_dyn_smem(gs_combine_kernel<E, KIND, STAGES>));
+    const unsigned g = wave_grid<gs_combine_kernel<E, KIND, STAGES>>(a.B.tiles, kStage + NV * kExp);
+    AFEM_LAUNCH((gs_combine_kernel<E, KIND, STAGES>), g, kRedThreads, kStage + a.nv * kExp, s, a);
     AFEM_CUDA_TRY(cudaGetLastError());
     return AFEM_OK;
+}
+// With four rows the exponents of 16 vectors take 64 KB beside the ring: its
+// depth leaves two blocks per SM.
+template <int E, int KIND>
+static int launch_gs_combine_e(const GsCombineArgs& a, cudaStream_t s) {
+    if constexpr (E == 4 && KIND != 0) {
+        if (a.nv > 14) return launch_gs_combine_s<E, KIND, 2, kMaxKrylov>(a, s);
+        if (a.nv > 11) return launch_gs_combine_s<E, KIND, 3, 14>(a, s);
+        return launch_gs_combine_s<E, KIND, 4, 11>(a, s);
+    } else {
+        return launch_gs_combine_s<E, KIND, 4, kMaxKrylov>(a, s);
+    }
 }
 template <int KIND>
 static int launch_gs_combine(int E, const GsCombineArgs& a, cudaStream_t s) {
@@ -1264,7 +1326,7 @@ int arnoldi_reserve(afem_mesh* m, int n, int mk, ArnoldiWork& w) {
     const int64_t tile = int64_t(w.rows) * (kRedThreads / n);
     w.B.tiles = (m->dev.n_master + tile - 1) / tile;
     w.B.stride = w.B.tiles * w.rows * kRedThreads;
-    w.B.estride = w.B.tiles * kRedThreads;
+    w.B.estride = w.B.tiles * kRedThreads * exp_words(w.rows);
     auto carve = [&](Carver& cv) {
         w.B.V = cv.take<int4>(size_t(mk + 1) * w.B.stride);
         w.B.e = cv.take<int>(size_t(mk + 1) * w.B.estride);

@@ -21,12 +21,12 @@ constexpr int kResErr = kResCol + kLadder * kMaxKrylov;
 constexpr int kResFlag = kResErr + kLadder;   // .x != 0: a G cell pass gave up waiting for a block copy
 constexpr int kResSize = kResFlag + 1;
 
-// The Krylov basis as integers on per-group exponents (see gs_dots_kernel).
+// The Krylov basis as integers, each complex entry with its exponent (see gs_dots_kernel).
 struct KrylovBasis {
     int4* V;          // [m+1][tiles][rows per thread][threads]
-    int* e;           // [m+1][tiles][threads]
-    int64_t stride;   // elements of a vector
-    int64_t estride;  // exponents of a vector
+    int* e;           // [m+1][tiles][threads][1 or 2 words] exponents, 16 bits per row
+    int64_t stride;   // entries of a vector
+    int64_t estride;  // exponent words of a vector
     int64_t tiles;
 };
 

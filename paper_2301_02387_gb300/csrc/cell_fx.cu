@@ -116,6 +116,13 @@ static FxBasis make_fx_basis(int p) {
     return f;
 }
 
+// Formed with the first launch of a degree (software arithmetic on an arm64 host).
+template <int P>
+static const FxBasis& fx_basis() {
+    static const FxBasis f = make_fx_basis(P);
+    return f;
+}
+
 constexpr int kFxColumns = 16;   // real columns of a block at most
 
 // Shared memory of cpb cells and nc columns (fields: with mean fields).
@@ -340,9 +347,9 @@ static int launch_p(const afem_mesh* m, const CellArgs& a, const double* x, cons
     const int block = std::min(256, (rows * nc + 31) / 32 * 32);
     const size_t smem = cell_fx_smem(NN, cpb, nc, PT == 2);
     AFEM_CUDA_TRY(allow_dyn_smem(cell_fx_kernel<P, PT>));
-    const FxBasis D = make_fx_basis(P);
     const dim3 grid(unsigned((ncell + cpb - 1) / cpb), unsigned((ncol + kFxColumns - 1) / kFxColumns));
-    AFEM_LAUNCH((cell_fx_kernel<P, PT>), grid, block, smem, s, a, D, x, U, y, ncol, cpb, ncell);
+    AFEM_LAUNCH((cell_fx_kernel<P, PT>), grid, block, smem, s, a, fx_basis<P>(), x, U, y, ncol, cpb,
+                ncell);
     AFEM_CUDA_TRY(cudaGetLastError());
     return AFEM_OK;
 }

@@ -591,6 +591,11 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_dots_kernel(const __grid_co
                 for (int r = 0; r < E; ++r) u[r] = s_v[(slot * E + r) * kRedThreads + tid];
                 int er[E], eu = 0;
                 read_exps<E>(s_ve + (slot * kRedThreads + tid) * EW, er);
+                if (k0 + (E - 1) * rc.R >= n_int) {   // surface rows (m w = 0) may hold anything
+#pragma unroll
+                    for (int r = 0; r < E; ++r)
+                        if (k0 + r * rc.R >= n_int) er[r] = 0;
+                }
 #pragma unroll
                 for (int r = 0; r < E; ++r) eu = max(eu, er[r]);
                 slot = slot + 1 == STAGES ? 0 : slot + 1;
@@ -903,7 +908,7 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_combine_kernel(const __grid
             eo[r] = bits ? bits + EM[r] - 1079 : 0;
             if (EM[r] > kFxMaxSum || eo[r] > kFxNan) eo[r] = kFxNan;
             if (eo[r] < kFxMinExp) eo[r] = 0;
-            top = max(top, eo[r]);
+            if (k0 + r * rc.R < n_int) top = max(top, eo[r]);   // (surface rows have no part in the norm)
             // t 2^(EM - 2101) = X 2^(eo - 1082), X = t 2^(60 - bits)
             const long long vx = eo[r] != 0 ? (tx[r] << (63 - bits)) >> 3 : 0, vy = eo[r] != 0 ? (ty[r] << (63 - bits)) >> 3 : 0;
             if (k0 + r * rc.R < N) {
@@ -922,7 +927,7 @@ __global__ void __launch_bounds__(kRedThreads, 2) gs_combine_kernel(const __grid
         write_exps<E>(eg + dst * a.B.estride, eo);
 #pragma unroll
         for (int r = 0; r < E; ++r) {
-            const int d = min(top - eo[r], 63);
+            const int d = min(max(top - eo[r], 0), 63);
             const Fx fx = fx_split(tx[r] >> d), fy = fx_split(ty[r] >> d);
             FxAcc sq{0, 0};
             fx_mad(sq, fx, fx);

@@ -105,3 +105,18 @@ def test_zero_columns_and_non_finite_entries(value, precision):
         phi[gm.n_interior // 2, 3] = value
         with pytest.raises(pkg.AfemError):
             pkg.arnoldi_step(gm, phi, None, 6, 0.01, precision=precision)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("value", [1e30, np.inf, np.nan])
+def test_surface_rows_may_hold_anything(value, precision):
+    """The orbitals vanish on the surface: what its rows hold has no part in the result inside
+    (two propagations of the same orbitals differ by the order of the scatter's additions)."""
+    import torch
+    import paper_2301_02387_gb300 as pkg
+    gm, om, op, perm = _space(36)
+    phi = torch.from_numpy(_orbitals(om, 7, 1)[perm]).cuda()
+    a = pkg.arnoldi_step(gm, phi, None, 6, 0.01, precision=precision)[0][:gm.n_interior].clone()
+    phi[gm.n_interior:] = value
+    b = pkg.arnoldi_step(gm, phi, None, 6, 0.01, precision=precision)[0][:gm.n_interior]
+    assert float((a - b).norm() / a.norm()) < (1e-13, 1e-6)[precision]

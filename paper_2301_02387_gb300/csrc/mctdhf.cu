@@ -651,11 +651,9 @@ static void finalize_cpartials(const double2* partial, int nblk, int k, double2*
 __global__ void csum_blocks_kernel(const double2* __restrict__ partial, int nblk, int k, double2* __restrict__ out) {
     for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < k; o += gridDim.x * blockDim.x) {
         double x = 0.0, y = 0.0;
-#pragma unroll 8
-        for (int b = 0; b < nblk; ++b) {   // (loads of eight rows in flight)
-            const double2 v = partial[int64_t(b) * k + o];
-            x += v.x;
-            y += v.y;
+        for (int b = 0; b < nblk; ++b) {
+            x += partial[int64_t(b) * k + o].x;
+            y += partial[int64_t(b) * k + o].y;
         }
         out[o] = make_double2(x, y);
     }

@@ -48,11 +48,13 @@
 namespace afem {
 
 // D = W^-1 Khat, each row on the scale of its largest entry (biased exponent e).
+template <int P>
 struct FxBasis {
-    int h[kMaxP1 * kMaxP1], l[kMaxP1 * kMaxP1];
-    int l8[kMaxP1 * kMaxP1];   // l / 8, for the products of low words
-    int e[kMaxP1];
-    double w3[kMaxP1 * kMaxP1 * kMaxP1], w3_lo[kMaxP1 * kMaxP1 * kMaxP1];   // w_a w_b w_c as a sum of two
+    static constexpr int P1 = P + 1;
+    int h[P1 * P1], l[P1 * P1];
+    int l8[P1 * P1];   // l / 8, for the products of low words
+    int e[P1];
+    double w3[P1 * P1 * P1], w3_lo[P1 * P1 * P1];   // w_a w_b w_c as a sum of two
 };
 
 // From the closed forms of the Gauss-Lobatto points and weights in long double, as
@@ -61,9 +63,10 @@ struct FxBasis {
 // 8.7e-16; as FP64 multiply-adds 1.1, 1.6, 4.3 and 8.6e-16).  H1 without potential:
 // 1.2, 1.6, 1.8 and 1.0e-16 (FP64 multiply-adds 1.2, 1.3, 1.7 and 4.6e-16): what is
 // left is the rounding of the lumped mass, the same in every cell of a size.
-static FxBasis make_fx_basis(int p) {
-    const long double z = p == 3 ? std::sqrt(0.2L) : std::sqrt(3.0L / 7.0L);   // the inner points on [-1, 1]
-    const int p1 = p + 1;
+template <int P>
+static FxBasis<P> make_fx_basis() {
+    const long double z = P == 3 ? std::sqrt(0.2L) : std::sqrt(3.0L / 7.0L);   // the inner points on [-1, 1]
+    constexpr int p = P, p1 = P + 1;
     long double x[kMaxP1] = {}, w[kMaxP1] = {};
     x[0] = -1.0L;
     x[p] = 1.0L;
@@ -87,7 +90,7 @@ static FxBasis make_fx_basis(int p) {
             d[q][q] -= r;
         }
     }
-    FxBasis f{};
+    FxBasis<P> f{};
     for (int i = 0; i < p1; ++i) {
         long double D[kMaxP1], top = 0.0L;
         for (int j = 0; j < p1; ++j) {
@@ -118,8 +121,8 @@ static FxBasis make_fx_basis(int p) {
 
 // Formed with the first launch of a degree (software arithmetic on an arm64 host).
 template <int P>
-static const FxBasis& fx_basis() {
-    static const FxBasis f = make_fx_basis(P);
+static const FxBasis<P>& fx_basis() {
+    static const FxBasis<P> f = make_fx_basis<P>();
     return f;
 }
 
@@ -136,10 +139,11 @@ static size_t cell_fx_smem(int nn, int cpb, int nc, bool fields) {
 constexpr int kSumInf = 0x7F00, kSumMinusInf = 0x7F01, kSumNan = 0x7F02;
 
 // Row i of D on a line with an infinity or NaN: which of the three the sum is.
-__device__ __noinline__ int non_finite_sum(const double* u, int step, const FxBasis& D, int p1, int i) {
+template <int P>
+__device__ __noinline__ int non_finite_sum(const double* u, int step, const FxBasis<P>& D, int i) {
     double f = 0.0;
-    for (int j = 0; j < p1; ++j)
-        f = fma(fma(double(D.h[i * p1 + j]), 4294967296.0, double(D.l[i * p1 + j])), u[j * step], f);
+    for (int j = 0; j <= P; ++j)
+        f = fma(fma(double(D.h[i * (P + 1) + j]), 4294967296.0, double(D.l[i * (P + 1) + j])), u[j * step], f);
     return f > 0.0 ? kSumInf : f < 0.0 ? kSumMinusInf : kSumNan;
 }
 
@@ -159,7 +163,7 @@ __device__ __forceinline__ double mean_field_part(double2 w, double2 u, int odd,
 // doubles; blockIdx.y selects kFxColumns of them.
 template <int P, int PT>
 __global__ void __launch_bounds__(256, PT == 2 ? 4 : 3) cell_fx_kernel(const __grid_constant__ CellArgs a,
-                                                      const __grid_constant__ FxBasis D, const double* __restrict__ x,
+                                                      const __grid_constant__ FxBasis<P> D, const double* __restrict__ x,
                                                       const double2* __restrict__ U, double* __restrict__ y, int ncol,
                                                       int cpb, int64_t ncell) {
     constexpr int P1 = P + 1, NN = P1 * P1 * P1, NP = P1 * P1;
@@ -297,7 +301,7 @@ __global__ void __launch_bounds__(256, PT == 2 ? 4 : 3) cell_fx_kernel(const __g
                 if constexpr (P == 4) acc.x += low >> 29;
                 long long t = (acc.hh << 4) + (acc.x >> 28);
                 int E = e ? e + D.e[i] - off : 0;   // the sum is t 2^(E - 2104)
-                if (e == 0x7FF) E = non_finite_sum(s_u + base, step, D, P1, i);
+                if (e == 0x7FF) E = non_finite_sum<P>(s_u + base, step, D, i);
                 const int o = base + i * step;
                 if (dir > 0) {
                     const int E1 = s_x[o], M = max(E, E1);
@@ -346,7 +350,7 @@ static int launch_p(const afem_mesh* m, const CellArgs& a, const double* x, cons
     const int rows = (cpb * P1 * P1 + rounds - 1) / rounds;
     const int block = std::min(256, (rows * nc + 31) / 32 * 32);
     const size_t smem = cell_fx_smem(NN, cpb, nc, PT == 2);
-    AFEM_CUDA_TRY(allow_dyn_smem(cell_fx_kernel<P, PT>));
+    if (smem > 48 * 1024) AFEM_CUDA_TRY(allow_dyn_smem(cell_fx_kernel<P, PT>));
     const dim3 grid(unsigned((ncell + cpb - 1) / cpb), unsigned((ncol + kFxColumns - 1) / kFxColumns));
     AFEM_LAUNCH((cell_fx_kernel<P, PT>), grid, block, smem, s, a, fx_basis<P>(), x, U, y, ncol, cpb,
                 ncell);

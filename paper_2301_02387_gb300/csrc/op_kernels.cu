@@ -15,8 +15,8 @@
 //
 // The unscaled length-gauge operators (the stiffness, H1~ and G) run in
 // cell_fx_kernel, their contractions on the integer pipe; the kernels here carry
-// the velocity gauge, the complex scaling and the pointwise-only operators, with
-// FP64 multiply-adds.
+// the velocity gauge, the complex scaling, the pointwise-only operators and one
+// or two real columns on small meshes, with FP64 multiply-adds.
 #include <cmath>
 
 #include "afem_internal.h"
@@ -248,6 +248,32 @@ __global__ void __launch_bounds__(256) g_cell_kernel(CellArgs a, const double2* 
 int launch_cell_fx(const afem_mesh* m, const CellArgs& a, const double* x, const double2* U, double* y, int ncol,
                    cudaStream_t s);
 
+template <typename T>
+static int launch_cell_op(const afem_mesh* m, const CellArgs& a, const T* x, T* y, int nv, cudaStream_t s);
+
+// y += A x or H1~ x (a.with_pot) on ncol real columns, plus the mean fields of G when U is given.
+// One or two columns on small meshes run as FP64 multiply-adds, a node per
+// thread: few threads hold a line each there, and the chain of a line's conversions
+// is longer than the p + 1 multiply-adds it replaces.  One column, FP64 and
+// integers in us: degree 2, 910 / 2,288 cells 12.5 and 16.3 / 16.4 and 16.4; degree
+// 3, 910 / 3,998 cells 14.2 and 24.6 / 24.6 and 27.7 (5,760: 34.9 and 34.5); degree
+// 4, 910 / 3,998 cells 21.7 and 30.9 / 37.3 and 38.7; two columns (H1), degree 2,
+// 910 / 1,296 cells 17.1 and 20.1 / 20.3 and 20.0; degree 4, 216 / 910 cells 17.1
+// and 22.4 / 39.1 and 38.8.
+static int launch_cell64(const afem_mesh* m, const CellArgs& a, const double* x, const double2* U, double* y, int ncol,
+                         cudaStream_t s) {
+    const int64_t cells = m->dev.ncell;
+    const int p = m->dev.p;
+    if (!U && ncol == 1 && cells < (p == 4 ? 3072 : p == 3 ? 4096 : p == 2 ? 1536 : 0))
+        return launch_cell_op<double>(m, a, x, y, 1, s);
+    if (!U && ncol == 2 && p >= 2 && cells < (p == 4 ? 512 : 1024)) {
+        if (a.with_pot)
+            return launch_cell_op<double2>(m, a, reinterpret_cast<const double2*>(x), reinterpret_cast<double2*>(y), 1, s);
+        return launch_cell_op<double>(m, a, x, y, 2, s);
+    }
+    return launch_cell_fx(m, a, x, U, y, ncol, s);
+}
+
 // velocity != 0: E holds the vector potential A of the velocity gauge (the
 // field term is then -i A . grad instead of E . r).
 int launch_g_cell(const afem_mesh* m, const double* E, const double2* v, const double2* U, double2* z, int n,
@@ -271,7 +297,7 @@ int launch_g_cell(const afem_mesh* m, const double* E, const double2* v, const d
     AFEM_CUDA_TRY(cudaMemsetAsync(z, 0, size_t(m->dev.n_master) * n * sizeof(double2), s));
     if (grid == 0) return AFEM_OK;
     if (!a.vg && !m->ecs_on)   // length gauge, unscaled: contractions on the integer pipe
-        return launch_cell_fx(m, a, reinterpret_cast<const double*>(v), U, reinterpret_cast<double*>(z), 2 * n, s);
+        return launch_cell64(m, a, reinterpret_cast<const double*>(v), U, reinterpret_cast<double*>(z), 2 * n, s);
     switch (p) {
 #define AFEM_CASE(PP)                                                                          \
     case PP: {                                                                                 \
@@ -386,7 +412,7 @@ int launch_stiffness(const afem_mesh* m, const double* x, double* y, int nv, int
     a.with_pot = 0;
     a.masked = masked;
     if (!y_zero) AFEM_CUDA_TRY(cudaMemsetAsync(y, 0, size_t(m->dev.n_master) * nv * sizeof(double), s));
-    return launch_cell_fx(m, a, x, nullptr, y, nv, s);
+    return launch_cell64(m, a, x, nullptr, y, nv, s);
 }
 
 int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int masked, cudaStream_t s,
@@ -406,8 +432,8 @@ int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void
         auto* yy = static_cast<double2*>(y);
         AFEM_CUDA_TRY(cudaMemsetAsync(yy, 0, size_t(N) * nv * sizeof(double2), s));
         int rc = m->ecs_on ? launch_cell_op<double2>(m, a, static_cast<const double2*>(x), yy, nv, s)
-                           : launch_cell_fx(m, a, static_cast<const double*>(x), nullptr, static_cast<double*>(y),
-                                            2 * nv, s);
+                           : launch_cell64(m, a, static_cast<const double*>(x), nullptr, static_cast<double*>(y),
+                                           2 * nv, s);
         if (rc) return rc;
         return launch_scale_rows<double2>(yy, m->dev.ml_inv, N, nv, s);
     }
@@ -431,7 +457,7 @@ int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void
         a.masked = 0;
         auto* yy = static_cast<double*>(y);
         AFEM_CUDA_TRY(cudaMemsetAsync(yy, 0, size_t(N) * nv * sizeof(double), s));
-        return launch_cell_fx(m, a, static_cast<const double*>(x), nullptr, yy, nv, s);
+        return launch_cell64(m, a, static_cast<const double*>(x), nullptr, yy, nv, s);
     }
     if (kind == AFEM_OP_POS || kind == AFEM_OP_FORCE) {   // y = M_L^-1 F[e.r] x or M_L^-1 F[e.force] x, masked
         a.c_kin = 0.0;

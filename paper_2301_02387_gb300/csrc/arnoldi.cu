@@ -31,9 +31,6 @@
 
 namespace afem {
 
-__device__ __forceinline__ double2 to_d2(double2 v) { return v; }
-__device__ __forceinline__ double2 to_d2(float2 v) { return make_double2(v.x, v.y); }
-
 // S[a][b] = sum_k w_k conj(A[k][a]) B[k][b] over rows k < n_rows (w_k = 1 when
 // w is null), reduced in the same launch: partial rows of 2*kout doubles (re,
 // im interleaved); the last block writes out[kout].  diag != 0: only a == b
@@ -43,8 +40,7 @@ __device__ __forceinline__ double2 to_d2(float2 v) { return make_double2(v.x, v.
 // on 102,533 rows took 27 us with four blocks per SM and one row at a time, 19 us
 // with two, 18 us with one.
 constexpr int kDotRows = 4;
-template <typename TB>
-__global__ void __launch_bounds__(kRedThreads) cdot_fused_kernel(const double2* __restrict__ A, int na, const TB* __restrict__ B, int nb,
+__global__ void __launch_bounds__(kRedThreads) cdot_fused_kernel(const double2* __restrict__ A, int na, const double2* __restrict__ B, int nb,
                                   const double* __restrict__ w, int64_t n_rows, int diag, double* __restrict__ partial,
                                   unsigned* __restrict__ counter, double2* __restrict__ out) {
     __shared__ double sx[kRedThreads], sy[kRedThreads];
@@ -65,7 +61,7 @@ __global__ void __launch_bounds__(kRedThreads) cdot_fused_kernel(const double2* 
                 u[q] = v[q] = make_double2(0.0, 0.0);
                 if (k < n_rows) {
                     u[q] = A[k * na + ia];
-                    v[q] = to_d2(B[k * nb + ib]);
+                    v[q] = B[k * nb + ib];
                     if (w) {
                         const double wk = w[k];
                         u[q] = make_double2(wk * u[q].x, wk * u[q].y);
@@ -1146,18 +1142,12 @@ __global__ void hang_rows32_kernel(const float2* __restrict__ U, const int32_t* 
     }
 }
 
-template <typename TB>
-int cdot_t(const double2* A, int na, const TB* B, int nb, const double* w, int64_t rows, int diag,
-           double2* partial, double2* out, unsigned* counter, cudaStream_t s) {
-    AFEM_LAUNCH((cdot_fused_kernel<TB>), row_blocks(rows, diag ? na : na * nb), kRedThreads, 0, s, A, na, B, nb, w, rows, diag,
+int cdot(const double2* A, int na, const double2* B, int nb, const double* w, int64_t rows, int diag,
+         double2* partial, double2* out, unsigned* counter, cudaStream_t s) {
+    AFEM_LAUNCH((cdot_fused_kernel), row_blocks(rows, diag ? na : na * nb), kRedThreads, 0, s, A, na, B, nb, w, rows, diag,
                 reinterpret_cast<double*>(partial), counter, out);
     AFEM_CUDA_TRY(cudaGetLastError());
     return AFEM_OK;
-}
-
-int cdot(const double2* A, int na, const double2* B, int nb, const double* w, int64_t rows, int diag,
-         double2* partial, double2* out, unsigned* counter, cudaStream_t s) {
-    return cdot_t<double2>(A, na, B, nb, w, rows, diag, partial, out, counter, s);
 }
 
 __global__ void to_c64_kernel(const double2* __restrict__ x, float2* __restrict__ y, int64_t n) {

@@ -1,8 +1,8 @@
 // Sums of float64 products on the integer pipe (block fixed point).
 //
 // GB300 issues FP64 multiply-adds at 2 per clock and SM (0.63 T/s measured
-// over the chip) and 32 x 32 + 64-bit integer multiply-adds (IMAD.WIDE) at 33
-// (9.8 T/s).  A float64 factor becomes a signed 60-bit integer on the scale of
+// over the chip) and 32 x 32 + 64-bit integer multiply-adds (IMAD.WIDE) at 31
+// (9.2 T/s).  A float64 factor becomes a signed 60-bit integer on the scale of
 // the largest factor of its group, X = v 2^(1082 - e) truncated, e the largest
 // biased exponent of the group (|X| < 2^60), split X = h 2^32 + l with both
 // words signed.  A product then costs three IMAD.WIDE,
@@ -10,12 +10,14 @@
 // into two 64-bit accumulators; the last term, below 2^62, is dropped: it is
 // 2^-58 of the largest product of the group, the truncation of the factors
 // 2^-59.  A chain of FP64 multiply-adds rounds at 2^-53 of its running value in
-// every step.  A group is the few values that a thread holds at a time, so the
-// scale follows the data from point to point.
+// every step.  A group is the few values that a thread holds at a time: the values of a
+// line of cell nodes, the rows of one sum.  Within it an error is bounded by the
+// group's largest, so a group never spans results of their own.
 //
-// Values below 2^-959 (biased exponent under 64) count as zero next to the
-// others of their group; groups with an infinity or NaN, or whose products
-// leave the float64 range, give NaN.
+// Values below 2^-959 (biased exponent under 64) lose bits and count as zero below
+// 2^-1018, except in the cell pass, which scales such lines up; groups with an
+// infinity or NaN, or whose products leave the float64 range, give NaN (the cell
+// pass: what FP64 gives).
 #pragma once
 
 #include <cuda_runtime.h>

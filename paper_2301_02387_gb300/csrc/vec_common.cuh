@@ -50,24 +50,6 @@ __device__ __forceinline__ float narrow_f64(double d) {
     if (rest > 0x10000000u || (rest == 0x10000000u && (keep & 1u))) r += 1u;
     return __uint_as_float(sign | r);
 }
-// narrow_f64(d * 2^k) with k added to the exponent field before rounding (no
-// floating-point multiply); zeros, infinities and NaNs as in narrow_f64.
-__device__ __forceinline__ float narrow_f64_scaled(double d, int k) {
-    const uint64_t b = static_cast<uint64_t>(__double_as_longlong(d));
-    const uint32_t sign = uint32_t(b >> 32) & 0x80000000u;
-    const int e = int((b >> 52) & 0x7FFull);
-    const uint64_t m = b & 0xFFFFFFFFFFFFFull;
-    if (e == 0x7FF) return __uint_as_float(sign | 0x7F800000u | (m ? 0x400000u : 0u));
-    if (e == 0) return __uint_as_float(sign);
-    const int ef = e - 896 + k;
-    if (ef <= 0) return __uint_as_float(sign);
-    if (ef >= 255) return __uint_as_float(sign | 0x7F800000u);
-    const uint32_t keep = uint32_t(m >> 29);
-    const uint32_t rest = uint32_t(m & 0x1FFFFFFFull);
-    uint32_t r = (uint32_t(ef) << 23) | keep;
-    if (rest > 0x10000000u || (rest == 0x10000000u && (keep & 1u))) r += 1u;
-    return __uint_as_float(sign | r);
-}
 // widen_f32(f) * 2^k through the exponent field: exact unless the result
 // leaves the binary64 normal range (zero or infinity then).
 __device__ __forceinline__ double widen_f32_scaled(float f, int k) {

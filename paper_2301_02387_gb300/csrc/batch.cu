@@ -5,6 +5,7 @@
 // the batch itself.  Each instance computes exactly what afem_op_apply
 // computes for it (Sec. 3.1, Eq. discretized_eom); only the scheduling is
 // shared.
+#include <algorithm>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -264,15 +265,20 @@ int afem_batch_op_apply(afem_batch* b, int kind, const double* E, void* const* x
         item0 += batch32_items(p[i], L4[i], b->meshes[i]->dev.ncell);
     }
     b->total_items = item0;
+    // the per-instance graph holds the buffers and fields (which the instance
+    // table does not have where the values are not whole quads)
+    const std::vector<double> fields(E ? E : nullptr, E ? E + 3 * count : nullptr);
+    if (b->block == 0 && b->exec &&
+        (!std::equal(x, x + count, b->cur_x.begin()) || !std::equal(y, y + count, b->cur_y.begin()) ||
+         fields != b->cur_E))
+        drop_graph(b);
     b->cur_x.assign(x, x + count);
     b->cur_y.assign(y, y + count);
     b->cur_n.assign(n_vec, n_vec + count);
-    if (E) b->cur_E.assign(E, E + 3 * count);
-    else b->cur_E.clear();
+    b->cur_E = fields;
     // upload the instance table only when it changed; the pinned staging copy is
     // rewritten only after the previous upload has been consumed
     if (staged != b->last) {
-        if (b->block == 0) drop_graph(b);   // the per-instance graph holds the buffers and fields
         AFEM_CUDA_TRY(cudaStreamSynchronize(s));
         std::memcpy(b->h_inst, staged.data(), staged.size());
         AFEM_CUDA_TRY(cudaMemcpyAsync(b->d_inst, b->h_inst, staged.size(), cudaMemcpyHostToDevice, s));

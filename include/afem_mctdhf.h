@@ -192,8 +192,9 @@ int afem_mesh_destroy(afem_mesh* mesh);
 /* Kernel-shape options of a mesh (library tuning; no counterpart in the paper).
  * AFEM_OPT_CELL32_VARIANT selects the float32 cell pass: 0 (default) sweeps the
  * lines of a cell with the 1D matrix in constant memory (afem_op_apply and the
- * smoothers) or computes each output node in one thread (the propagators' G, and
- * the CG sweeps' stiffness with p.Ap), 1 computes the 1D contractions
+ * smoothers, but for small meshes and short rows) or computes each output node in
+ * one thread (there, in the propagators' G, and in the CG sweeps' stiffness with
+ * p.Ap), 1 computes the 1D contractions
  * line by line with direction-wise accumulation in shared memory, 2 does the
  * same for the stiffness with one thread per (line, column pair) and the 1D
  * matrix in registers (1, 2 or 4 column quads; other passes as for 0).  All
@@ -629,8 +630,9 @@ int afem_tdse_vjp(afem_mesh* mesh, const double* e_dir, const double* E, int n_s
  * signature times candidate schedules on the batch itself -- the persistent
  * launch with grids of 2 or all resident blocks per SM at 256 and 128
  * threads or one block per work item, and the instances' own passes on 4, 8
- * or 16 parallel streams (reported as block 0, grid = streams) -- and keeps
- * the fastest (afem_batch_get_tuning).  With
+ * or 16 parallel streams (reported as block 0, grid = streams), in the faster
+ * of two forms of the cell pass -- and keeps the fastest
+ * (afem_batch_get_tuning).  With
  * AFEM_BATCH_GRAPH the zero, cell and scale passes are captured once into a
  * CUDA graph on a private stream and replayed on `stream`; the per-instance
  * table (pointers, fields) lives in device memory and is re-uploaded when

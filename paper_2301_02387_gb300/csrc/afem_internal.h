@@ -189,8 +189,10 @@ struct afem_mesh {
 namespace afem {
 int upload_mesh(afem_mesh* m);
 void free_device_mesh(DeviceMesh& d);
+// Forms of the float32 cell passes: a thread per node, line sweeps, or by size.
+enum class CellForm { kNode, kLines, kBySize };
 int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void* y, int nvec,
-                    cudaStream_t s);
+                    cudaStream_t s, CellForm form = CellForm::kBySize);
 // y = A x (y_zero: y is already cleared)
 int launch_stiffness(const afem_mesh* m, const double* x, double* y, int nv, int masked, cudaStream_t s,
                      bool y_zero = false);

@@ -1186,7 +1186,8 @@ int to_c64(const double2* x, float2* y, int64_t n, cudaStream_t s) {
 }
 
 int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const float2* U, float2* z, int n,
-                    cudaStream_t s, int velocity, const float2* U_hang = nullptr, bool lines = false);
+                    cudaStream_t s, int velocity, const float2* U_hang = nullptr,
+                    CellForm form = CellForm::kNode);
 
 // Blocks of kernel K for `tiles` tiles: one resident wave at most (every block
 // then takes several tiles and adds one row of partial sums).

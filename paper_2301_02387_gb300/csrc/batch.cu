@@ -52,6 +52,7 @@ struct afem_batch {
     int sig_kind = -1;
     std::vector<int> sig_L4;
     int block = 0, grid = 0, per_sm = 0;
+    CellForm form = CellForm::kLines;   // of the per-instance passes
     size_t smem = 0;
     std::vector<double> cand_ms;
     std::vector<int> cand_block, cand_grid;
@@ -77,7 +78,7 @@ int launch_per_instance(afem_batch* b, int kind, int streams, cudaStream_t s) {
     for (int i = 0; i < count; ++i) {
         const double* E = b->cur_E.empty() ? nullptr : b->cur_E.data() + 3 * i;
         int rc = launch_op_apply(b->meshes[i], kind, E, b->cur_x[i], b->cur_y[i], b->cur_n[i],
-                                 b->par[i % streams]);
+                                 b->par[i % streams], b->form);
         if (rc) return rc;
     }
     for (int j = 0; j < streams; ++j) {
@@ -156,6 +157,7 @@ int tune(afem_batch* b, int kind, bool persistent, cudaStream_t s) {
             }
         }
     }
+    b->form = CellForm::kLines;
     for (int streams : {4, 8, 16}) {
         double ms = 0.0;
         int rc = time_shape(b, kind, 0, unsigned(streams), 0, s, &ms);
@@ -168,6 +170,20 @@ int tune(afem_batch* b, int kind, bool persistent, cudaStream_t s) {
             b->block = 0;
             b->grid = streams;
             b->per_sm = 0;
+        }
+    }
+    // side by side the two forms of the cell pass share the chip in another way than
+    // alone (8 uneven instances: line sweeps 162 us, by each one's size 173, a thread
+    // per node 245; three instances of 2,430 to 4,558 cells at degree 3: 34 and 32 us)
+    if (b->block == 0) {
+        double ms = 0.0;
+        b->form = CellForm::kNode;
+        if (int rc = time_shape(b, kind, 0, unsigned(b->grid), 0, s, &ms)) return rc;
+        if (ms < best) {
+            for (size_t i = 0; i < b->cand_ms.size(); ++i)
+                if (b->cand_block[i] == 0 && b->cand_grid[i] == b->grid) b->cand_ms[i] = ms;
+        } else {
+            b->form = CellForm::kLines;
         }
     }
     return AFEM_OK;

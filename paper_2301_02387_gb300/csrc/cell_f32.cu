@@ -1454,7 +1454,12 @@ static int launch_pencil_p(const afem_mesh* m, const CellArgs32& a, const float*
     constexpr int P1 = P + 1, NN = P1 * P1 * P1;
     const int groups = lanes / VEC, Q = std::min(groups, kPencilFloats / VEC);
     // whole cells per block: as many as give each thread one pencil per sweep
-    const int per = P1 * P1 * Q, cpb = std::max(1, std::min(16, 256 / per));
+    const int per = P1 * P1 * Q;
+    int cpb = std::max(1, std::min(16, 256 / per));
+    // one or two floats: fewer, where the blocks would be under four per SM (2 floats
+    // at degree 3, stiffness on 6,504 cells 18.5 -> 16.4 us, H1 on 910 cells 20.5 -> 17.6;
+    // wider rows gain as often as they lose)
+    if (lanes <= 2) cpb = std::max(1, std::min(cpb, int(a.ncell / (4 * device_sms()))));
     const int rounds = (cpb * per + 255) / 256;
     const int block = std::min(256, ((cpb * P1 * P1 + rounds - 1) / rounds * Q + 31) / 32 * 32);
     const size_t smem = size_t(cpb) * NN * (2 * Q * VEC * sizeof(float) + sizeof(float) + 2 * sizeof(int)) +
@@ -1490,30 +1495,32 @@ static int launch_pencil32(const afem_mesh* m, const CellArgs32& a, const float*
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Whether `lanes` floats per node run faster in the node-per-thread form: it has
+// Whether `lanes` floats per node run as line sweeps.  The node-per-thread form has
 // p + 1 times the threads, which counts while the line sweeps leave the chip
 // partly idle.  The lines lie where both took the same time; stiffness, node form
 // and line sweeps in us: 4 floats, degree 4, 910 / 6,504 / 12,902 cells 15.1 and
 // 24.5 / 22.7 and 27.1 / 30.9 and 31.1 (17,500: 45.6 and 42.9), degree 3, 910 /
-// 27,672 cells 12.9 and 18.1 / 30.8 and 35.0, degree 2, 18,304 cells 14.4 and 16.4;
+// 27,672 cells 12.9 and 18.1 / 30.8 and 35.0, degree 2, 18,304 / 27,672 cells 14.4 and 16.4 / 18.5
+// and 18.8 (H1 26.7 and 25.6);
 // 8 floats, degree 4, 2,288 / 8,728 cells 20.7 and 22.6 / 37.0 and 35.0; 16 floats, degree 4, 692 / 1,296
 // cells 18.5 and 20.6 / 24.7 and 23.7, degree 3, 1,296 / 6,504 cells 16.4 and 18.5
 // / 24.8 and 24.7; one float, degree 4, 1,296 / 3,998 cells 16.3 and 20.3 / 20.6
 // and 20.6, degree 3, 910 / 2,288 cells 12.6 and 16.4 / 14.4 and 14.1.
-static bool node_form32(const afem_mesh* m, int lanes, bool aligned) {
+static bool line_form32(const afem_mesh* m, int lanes, bool aligned, CellForm form) {
+    if (form != CellForm::kBySize) return form == CellForm::kLines;
     const int64_t cells = m->dev.ncell;
     const int p = m->dev.p;
-    if (lanes <= 2) return p >= 3 && cells < (p == 4 ? 3072 : 1536);
-    if (lanes % 4 != 0 || lanes > 16 || !aligned) return false;
-    if (lanes == 4) return p == 4 ? cells <= 16384 : p >= 2;
-    return cells * lanes < (p == 4 ? (lanes == 8 ? 32768 : 16384) : p == 3 ? 80000 : 0);
+    if (lanes <= 2) return p < 3 || cells >= (p == 4 ? 3072 : 1536);
+    if (lanes % 4 != 0 || lanes > 16 || !aligned) return true;
+    if (lanes == 4) return p == 4 ? cells > 16384 : p == 2 ? cells > 20480 : p == 1;
+    return cells * lanes >= (p == 4 ? (lanes == 8 ? 32768 : 16384) : p == 3 ? 80000 : 0);
 }
 
 // pap_slots (optional): [kPapSlots][nv] FP64 sums that receive p.Ap per column
 // (x = p, masked), for nv in {4, 8, 16} on the four-lane path; returns
 // AFEM_EINVAL when they are asked for outside it.
 int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int masked, cudaStream_t s,
-                       double* pap_slots, bool y_zero) {
+                       double* pap_slots, bool y_zero, CellForm form) {
     CellArgs32 a = make_cell_args32(m);
     a.masked = masked;
     a.y_zero = y_zero ? 1 : 0;
@@ -1524,7 +1531,7 @@ int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int
         a.pap_slots = pap_slots;
     }
     // p.Ap and the shape options stay with the node- and line-ordered forms
-    if (!pap_slots && m->cell32_variant == 0 && !node_form32(m, nv, aligned16(x) && aligned16(y)))
+    if (!pap_slots && m->cell32_variant == 0 && line_form32(m, nv, aligned16(x) && aligned16(y), form))
         return launch_pencil32<false>(m, a, x, y, nv, s);
     if (quads) return launch32v<false>(m, a, x, nullptr, y, nv, 0, s);
     return launch32<float, false>(m, a, x, nullptr, y, nv, s);
@@ -1532,13 +1539,13 @@ int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int
 
 // z = H1~ v + mean field (complex64), Dirichlet-masked.
 // velocity != 0: E holds the vector potential A (velocity gauge), applied by
-// the generic (two-lane) kernel.  lines: a single application, which may run as
-// line sweeps; the propagators' repeated ones keep the node-per-thread pass: the
+// the generic (two-lane) kernel.  form: a single application may run as line
+// sweeps; the propagators' repeated ones keep the node-per-thread pass: the
 // order of the scatter's additions decides rounding that adds up over a propagation,
 // and with it a dipole signal of five steps differs from run to run by 1e-8 of its
 // norm (one comparison of the sweeps against this pass showed 7e-8).
 int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const float2* U, float2* z, int n,
-                    cudaStream_t s, int velocity, const float2* U_hang, bool lines) {
+                    cudaStream_t s, int velocity, const float2* U_hang, CellForm form) {
     CellArgs32 a = make_cell_args32(m);
     a.masked = 1;
     a.u_hang = U ? U_hang : nullptr;
@@ -1556,7 +1563,7 @@ int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const 
         for (int i = 0; i < 3; ++i) a.Avec[i] = float(E[i]);
         return launch32<float2, true>(m, a, v, U, z, n, s);
     }
-    if (lines && !U && m->cell32_variant == 0 && !node_form32(m, 2 * n, aligned16(v) && aligned16(z)))
+    if (!U && m->cell32_variant == 0 && line_form32(m, 2 * n, aligned16(v) && aligned16(z), form))
         return launch_pencil32<true>(m, a, reinterpret_cast<const float*>(v), reinterpret_cast<float*>(z), 2 * n, s);
     if (n % 2 == 0 && aligned16(v) && aligned16(z))
         return launch32v<true>(m, a, reinterpret_cast<const float*>(v), U, reinterpret_cast<float*>(z), 2 * n, n, s);

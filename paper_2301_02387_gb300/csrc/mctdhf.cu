@@ -723,8 +723,6 @@ static int ci_sigma(const CiTables& t, const StepWork& w, const double2* v, doub
     return AFEM_OK;
 }
 
-int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void* y, int nvec, cudaStream_t s);
-
 int mctdhf_step(afem_mctdhf* S, double2* phi, double2* C, double* W, const double* E, double dt, double cg_rtol,
                 int cg_max_it, afem_step_info* info, cudaStream_t s) {
     afem_mesh* m = S->mesh;

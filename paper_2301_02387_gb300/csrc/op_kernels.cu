@@ -264,7 +264,7 @@ static int launch_cell64(const afem_mesh* m, const CellArgs& a, const double* x,
                          cudaStream_t s) {
     const int64_t cells = m->dev.ncell;
     const int p = m->dev.p;
-    if (!U && ncol == 1 && cells < (p == 4 ? 3072 : p == 3 ? 4096 : p == 2 ? 1536 : 0))
+    if (!U && ncol == 1 && cells < (p >= 3 ? 4096 : p == 2 ? 1536 : 0))
         return launch_cell_op<double>(m, a, x, y, 1, s);
     if (!U && ncol == 2 && p >= 2 && cells < (p == 4 ? 512 : 1024)) {
         if (a.with_pot)
@@ -416,12 +416,13 @@ int launch_stiffness(const afem_mesh* m, const double* x, double* y, int nv, int
 }
 
 int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int masked, cudaStream_t s,
-                       double* pap_slots = nullptr, bool y_zero = false);
+                       double* pap_slots = nullptr, bool y_zero = false, CellForm form = CellForm::kBySize);
 int launch_g_cell32(const afem_mesh* m, const double* E, const float2* v, const float2* U, float2* z, int n,
-                    cudaStream_t s, int velocity = 0, const float2* U_hang = nullptr, bool lines = false);
+                    cudaStream_t s, int velocity = 0, const float2* U_hang = nullptr,
+                    CellForm form = CellForm::kNode);
 
 int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void* y, int nv,
-                    cudaStream_t s) {
+                    cudaStream_t s, CellForm form) {
     CellArgs a = make_cell_args(m);
     const int64_t N = m->dev.n_master;
     if (kind == AFEM_OP_H1) {
@@ -471,10 +472,12 @@ int launch_op_apply(afem_mesh* m, int kind, const double* E, const void* x, void
         return launch_scale_rows<double2>(yy, m->dev.ml_inv, N, nv, s);
     }
     if (kind == AFEM_OP_STIFF_F32)
-        return launch_stiffness32(m, static_cast<const float*>(x), static_cast<float*>(y), nv, 0, s);
+        return launch_stiffness32(m, static_cast<const float*>(x), static_cast<float*>(y), nv, 0, s, nullptr, false,
+                                  form);
     if (kind == AFEM_OP_H1_C64 || kind == AFEM_OP_H1_VG_C64) {
         auto* yy = static_cast<float2*>(y);
-        int rc = launch_g_cell32(m, E, static_cast<const float2*>(x), nullptr, yy, nv, s, kind == AFEM_OP_H1_VG_C64, nullptr, true);
+        int rc = launch_g_cell32(m, E, static_cast<const float2*>(x), nullptr, yy, nv, s, kind == AFEM_OP_H1_VG_C64,
+                                 nullptr, form);
         if (rc) return rc;
         return launch_scale_rows<float2>(yy, m->dev.ml_inv, N, nv, s);
     }

@@ -40,7 +40,7 @@
 namespace afem {
 
 int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int masked, cudaStream_t s,
-                       double* pap_slots, bool y_zero = false);
+                       double* pap_slots, bool y_zero = false, CellForm form = CellForm::kBySize);
 int poisson_rhs_bc(afem_mesh* m, const double2* phi, int n, double* W, double* b, double* qpart, double* q,
                    cudaStream_t s);
 int mom_blocks_count();

@@ -980,7 +980,7 @@ __global__ void residual64_kernel(const double* __restrict__ b, const double* __
 }
 
 int launch_stiffness32(const afem_mesh* m, const float* x, float* y, int nv, int masked, cudaStream_t s,
-                       double* pap_slots = nullptr, bool y_zero = false);
+                       double* pap_slots = nullptr, bool y_zero = false, CellForm form = CellForm::kBySize);
 
 // Reliable-update form of the mixed solve: one continuous float32 CG per
 // column whose correction d is folded into the float64 W, and whose residual is

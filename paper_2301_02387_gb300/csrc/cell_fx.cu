@@ -33,7 +33,10 @@
 // Per node and column: 9 (p + 1) IMAD.WIDE (12 at degree 4; 31 per clock and SM),
 // three conversions to integers, one back and one FP64 multiply-add.  The
 // stiffness above takes 595 us; 9 columns at degree 3 on 4,164 cells 61 us instead
-// of 120.  What bounds it is instruction issue and the barriers between sweeps.
+// of 120, with the mean fields of 3 orbitals 71 us instead of 106.  Counters of the
+// first: 504 instructions per node and column, issue 53 %, multiply pipe 42 %, ALU
+// 38 %, FP64 pipe 27 %, DRAM 6 %; warps wait for the barriers between sweeps, for
+// instructions and for the multiply pipe.
 // The sums of the directions as FP64 numbers took longer (622 and 81 us): the
 // conversions run at 1.6 per clock and SM.
 #include <algorithm>
@@ -149,8 +152,9 @@ __device__ __noinline__ int non_finite_sum(const double* u, int step, const FxBa
 
 // One component of acc + w u: the real (odd = 0) or the imaginary part.  The
 // operands are selected, with the sign as a bit, so that lanes of both kinds
-// share the two multiply-adds (as two expressions a warp ran all four: 3 complex
-// orbitals at degree 3 on 4,164 cells took 82 us, now 66 us).
+// share the two multiply-adds (as two expressions a warp ran all four: the pass on 3
+// complex orbitals at degree 3 and 4,164 cells took 82 us in place of 66, in the
+// form of one scale per cell).
 __device__ __forceinline__ double mean_field_part(double2 w, double2 u, int odd, double acc) {
     const double same = odd ? u.y : u.x, other = odd ? u.x : u.y;
     const double signed_other =

@@ -19,7 +19,8 @@
 // columns (its FP64 sums then take 64 registers at 64 columns).  Every wait is
 // bounded; a block that gives up sets *status.  The tensor pipe is about 1 %
 // busy: what bounds the kernel is the instructions that stage, split and sum a
-// tile.  The orbital count is a compile-time constant for them: with divisions
+// tile, about 3,750 issue slots a scheduler and, at 64 columns, 8,192 FP64 additions
+// (3,900 clocks of that pipe) of the 9,600 clocks that a tile takes.  The orbital count is a compile-time constant for them: with divisions
 // by run-time counts, one warpgroup and half the warps in flight, 8 orbitals on
 // 2,647,013 points took 8.1 ms (26,200 warp instructions per tile), against 0.25
 // ms for the bytes; now 2.6 ms (15,000).

@@ -136,7 +136,12 @@ struct PointArgs {
 // one column), each thread 4 harmonics x 4 columns in registers.  As FP64
 // multiply-adds with both factors from shared memory, and divisions in the
 // harmonics, the 830,209 points x 16 columns of the H2 benchmark took 13.9 ms;
-// now 7.1 ms.
+// now 7.1 ms.  A moment is exact to 2^-58 of the tile's largest harmonic times its
+// largest density, which on a coarse tile can be far above the products themselves (up
+// to 1e-2 of a high moment); the surface data divide it by that power of the
+// surface's radius, where it is below 1e-16 of the monopole (meshes of 2 to 8
+// cells per axis, boxes of 16 to 80, Gaussians of exponent 0.05 to 2: 1e-17 to 1e-20,
+// float64 sums 4e-17 to 2e-15).
 constexpr int kMomLm4 = (kNlm + 3) / 4 * 4;   // harmonics padded to quads
 constexpr int kMomRow = kMomLm4 + 2;          // row of a point (8-byte words; even, off the bank period)
 static size_t mom_smem(int ncol) {
